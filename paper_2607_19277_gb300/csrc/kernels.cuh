@@ -54,6 +54,7 @@ struct StageArgs {
   PhysParamsT<float> ppf;
   float fa = 0.0f, fb = 0.0f;
   int combine = 0;
+  int zs = 0;                   // a work item is 16 >> zs planes of a block (stage_go's rule)
 };
 
 // Conserved + auxiliary values of the cell (x, y, z) of block b in the halo view: the
@@ -322,8 +323,9 @@ struct StageSmem {
 //   -- CTA barrier --
 //   D. flux divergence, SSPRK combine and store of cell (x, y, k);
 //   -- CTA barrier, with one flux buffer only: the next plane's faces overwrite it --
-// Raw planes arrive by TMA one or two planes ahead of their conversion.
-template <template <typename> class PT, typename R, int LIM, int FLUX, int MINB, int RAW, int SFB>
+// Raw planes arrive by TMA one or two planes ahead of their conversion. With Z_CUT the launch's
+// work items are parts of blocks (A.zs): the same planes, faces and cells, the same arithmetic.
+template <template <typename> class PT, typename R, int LIM, int FLUX, int MINB, int RAW, int SFB, bool Z_CUT>
 __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant__ CUtensorMap tmap,
                                                            StageArgs A) {
   static_assert(RAW >= 3 && RAW <= 5, "three to five raw slots");
@@ -339,8 +341,13 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   constexpr bool PAIRED = sizeof(R) == 4 && PairPhys<P>::OK && (FLUX == FLUX_HLL || FLUX == FLUX_TVDLF);
   constexpr int NAW = NA > 0 ? NA : 1;
   constexpr bool RESP = res_of<P>::value;   // resistive MHD sources
-  // completions of raw slot s's barrier per block (planes -2 .. 17 = TMA sequence 0 .. 19)
-  auto phases = [](int s) { return (20 + RAW - 1 - s) / RAW; };
+  // A work item is planes k0 .. k0 + nz - 1 of a block (the whole block for zs = 0): it reads
+  // planes k0 - 2 .. k0 + nz + 1, TMA sequence 0 .. nz + 3.
+  const int zs = Z_CUT ? A.zs : 0;
+  const int nz = NB >> zs;
+  const int nitem = A.nblk << zs;
+  // completions of raw slot s's barrier per item
+  auto phases = [nz](int s) { return (nz + 4 + RAW - 1 - s) / RAW; };
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
   R* sRaw = reinterpret_cast<R*>(smem_raw + S::raw);
@@ -386,8 +393,8 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   }
   __syncthreads();
   int st = 0;
-  // Persistent loop: this CTA starts with block blockIdx.x and then takes the next free block
-  // from the launch's counter; every block completes PHASES phases of each raw slot's barrier.
+  // Persistent loop: this CTA starts with item blockIdx.x and then takes the next free item
+  // from the launch's counter; every item completes phases(s) phases of raw slot s's barrier.
   __shared__ int s_next;
   __shared__ int s_src[6], s_slot[6];   // face sources / register slots of the current block
   __shared__ R s_kc[12];                // per-(solve, level) constants, formed by thread 0
@@ -414,8 +421,9 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   const R kap0 = R(A.htc_kappa0);
   const R reta = R(A.eta);
   R dxr[3] = {R(0), R(0), R(0)};
-  if (t == 0 && blockIdx.x < A.nblk) {
-    const int b0 = A.wl ? A.wl[blockIdx.x] : (int)blockIdx.x;
+  if (t == 0 && (int)blockIdx.x < nitem) {
+    const int i0 = (int)blockIdx.x >> zs;
+    const int b0 = A.wl ? A.wl[i0] : i0;
 #pragma unroll
     for (int f = 0; f < 6; ++f) {
       s_src[f] = A.bd[b0].src[f];
@@ -425,9 +433,11 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   __syncthreads();
   const int* src = s_src;
   const int* slot = s_slot;
-  // work item w is pool block b (the work list of a batch skips the blocks of detached solves)
-  for (int w = blockIdx.x, jb = 0; w < A.nblk; ++jb) {
-  const int b = A.wl ? A.wl[w] : w;
+  // work item w lies in pool block b (the work list of a batch skips the blocks of detached
+  // solves); the items of a block are consecutive
+  for (int w = blockIdx.x, jb = 0; w < nitem; ++jb) {
+  const int b = A.wl ? A.wl[w >> zs] : w >> zs;
+  const int k0 = (w & ((1 << zs) - 1)) * nz, k1 = k0 + nz;
   const int sv = A.solve_of ? A.solve_of[b] : 0;
   unsigned long long* speeds = A.speeds ? A.speeds + 2 * sv : nullptr;
   const BlockDesc& bd = A.bd[b];
@@ -472,13 +482,14 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
     key_lev = bd.level;
   }
 
-  // plane p (-2 .. 17) -> TMA sequence q = p + 2, raw slot q % RAW, phase (q / RAW) of this block
+  // plane p (k0 - 2 .. k1 + 1) -> TMA sequence q = p - k0 + 2, raw slot q % RAW, phase (q / RAW)
+  // of this item
   auto plane_tma = [&](int p) -> bool {   // does plane p come by TMA (else loaded directly)?
     if (p >= 0 && p < NB) return true;
     return src[p < 0 ? 4 : 5] >= 0;
   };
   auto issue = [&](int p) {               // thread 0 only
-    const int q = p + 2;
+    const int q = p - k0 + 2;
     uint64_t* br = bar + (q % RAW);
     if (plane_tma(p)) {
       int blk = b, z = p;
@@ -495,7 +506,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   auto ring = [&](int p) -> R* { return sP + (size_t)pslot(p) * NT * 400; };
   // Primitive recovery of this thread's own column at plane p into the primitive ring.
   auto convert_own = [&](int p) {
-    const int q = p + 2;
+    const int q = p - k0 + 2;
     R u[NT];
     if (plane_tma(p)) {
       if (!mbar_wait(bar + (q % RAW), ((q / RAW) + jb * phases(q % RAW)) & 1, WAIT_LIMIT)) st |= ST_ETIMEOUT;
@@ -616,53 +627,54 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
     riemann<P, R, 1, FLUX>(pl, pr, f, pp);
   };
 
-  // ---- prologue: raw planes by TMA, halo fetches of planes 0 and 1, primitives of planes
-  // -2 .. 1 of this column, the z-face at -1/2, the halo of plane 0
+  // ---- prologue: raw planes by TMA, halo fetches of planes k0 and k0 + 1, primitives of
+  // planes k0 - 2 .. k0 + 1 of this column, the z-face at k0 - 1/2, the halo of plane k0
   if (t == 0) {
-    fence_proxy_async();   // the previous block's reads of the ring precede these copies
-    for (int p = -2; p <= RAW - 3; ++p) issue(p);
+    fence_proxy_async();   // the previous item's reads of the ring precede these copies
+    for (int p = k0 - 2; p <= k0 + RAW - 3; ++p) issue(p);   // nz >= 1: at least RAW planes
   }
-  prefetch_halo(0);
-  prefetch_halo(1);
-  convert_own(-2);
-  convert_own(-1);
-  __syncthreads();   // raw slots of planes -2 and -1 are free
+  prefetch_halo(k0);
+  if (k0 + 1 < k1) prefetch_halo(k0 + 1);
+  convert_own(k0 - 2);
+  convert_own(k0 - 1);
+  __syncthreads();   // raw slots of planes k0 - 2 and k0 - 1 are free
   if (t == 0) {
     fence_proxy_async();
-    for (int p = RAW - 2; p <= (RAW == 3 ? 2 : 3); ++p) issue(p);
+    for (int p = RAW - 2; p <= (RAW == 3 ? 2 : 3); ++p)
+      if (p <= nz + 1) issue(k0 + p);
   }
-  convert_own(0);
+  convert_own(k0);
   R fzd[NV], fzu[NV], hz[NV];
-  {  // z-slope of plane -1 from planes -2, -1 and 0 ... before plane 1 takes plane -2's slot
-    const R* r0 = ring(-2) + cellp;
-    const R* r1 = ring(-1) + cellp;
-    const R* r2 = ring(0) + cellp;
+  {  // z-slope of plane k0 - 1 ... before plane k0 + 1 takes plane k0 - 2's slot
+    const R* r0 = ring(k0 - 2) + cellp;
+    const R* r1 = ring(k0 - 1) + cellp;
+    const R* r2 = ring(k0) + cellp;
 #pragma unroll
     for (int v = 0; v < NV; ++v)
       hz[v] = v < P::NREC ? half_slope<R, LIM>(r1[v * 400] - r0[v * 400], r2[v * 400] - r1[v * 400]) : R(0);
   }
-  convert_own(1);
-  zface(-1, fzd, hz);
-  if (FR && slot[4] >= 0) {
+  convert_own(k0 + 1);
+  zface(k0 - 1, fzd, hz);
+  if (FR && k0 == 0 && slot[4] >= 0) {
 #pragma unroll
     for (int v = 0; v < NV; ++v) FR[((size_t)slot[4] * NV + v) * 256 + cell2] = fzd[v];
   }
-  convert_halo(0);
-  __syncthreads();   // plane 0 of the ring (interior and halo) is complete
-  if (RAW == 3 && t == 0) {   // raw slots of planes 0 and 1, converted above
+  convert_halo(k0);
+  __syncthreads();   // plane k0 of the ring (interior and halo) is complete
+  if (RAW == 3 && t == 0) {   // raw slots of planes k0 and k0 + 1, converted above
     fence_proxy_async();
-    issue(3);
-    issue(4);
+    if (3 <= nz + 1) issue(k0 + 3);
+    if (4 <= nz + 1) issue(k0 + 4);
   }
 
   R ssum = R(0), smax = R(0);
 
   R Tkm1 = R(0);   // conduction: T = p / rho of this column at plane k - 1
   R Bkm1[3] = {R(0), R(0), R(0)};   // resistivity: B of this column at plane k - 1
-  for (int k = 0; k < NB; ++k) {
+  for (int k = k0; k < k1; ++k) {
     R* sFx = sFx0 + (SFB == 2 ? (k & 1) : 0) * NV * 272;
     R* sFy = sFy0 + (SFB == 2 ? (k & 1) : 0) * NV * 272;
-    if (RAW == 4 && t == 0 && k >= 1 && k + 3 <= NB + 1) {
+    if (RAW == 4 && t == 0 && k > k0 && k + 3 <= k1 + 1) {
       fence_proxy_async();
       issue(k + 3);   // raw slot of plane k-1, read by its update before the previous barrier
     }
@@ -676,9 +688,9 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
 #pragma unroll
       for (int i = 0; i < 3; ++i) Bkm1[i] = r[(P::BOFF + i) * 400];
     }
-    if (k + 2 <= NB + 1) convert_own(k + 2);
-    if (k + 1 < NB) convert_halo(k + 1);
-    if (k + 2 < NB) prefetch_halo(k + 2);
+    convert_own(k + 2);
+    if (k + 1 < k1) convert_halo(k + 1);
+    if (k + 2 < k1) prefetch_halo(k + 2);
     // ---- C
     const R* Ck = ring(k);
     // conduction target kappa0 T^(5/2) b.grad T of cell (tx, ty, k) (Eq. 10): central
@@ -833,11 +845,11 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
       }
     }
     __syncthreads();
-    if (RAW == 5 && t == 0 && k + 4 <= NB + 1) {
+    if (RAW == 5 && t == 0 && k + 4 <= k1 + 1) {
       fence_proxy_async();
       issue(k + 4);   // raw slot of plane k-1, whose update finished before this barrier
     }
-    if (RAW == 3 && t == 0 && k + 5 <= NB + 1) {
+    if (RAW == 3 && t == 0 && k + 5 <= k1 + 1) {
       fence_proxy_async();
       issue(k + 5);   // raw slot of plane k+2, converted by every thread before this barrier
     }
@@ -846,7 +858,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
       const size_t cell = (size_t)k * 256 + cell2;
       const size_t base = (size_t)b * NT * NCELL + cell;
       // U_s of the cell: the raw TMA slot, or global memory (layout with three slots)
-      const R* raw = US_GLOBAL ? Us + base : sRaw + (size_t)((k + 2) % RAW) * NT * 256 + cell2;
+      const R* raw = US_GLOBAL ? Us + base : sRaw + (size_t)((k - k0 + 2) % RAW) * NT * 256 + cell2;
       constexpr int RSTR = US_GLOBAL ? NCELL : 256;
       R out[NV];
       if constexpr (P::SOURCE) {
@@ -920,8 +932,8 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
     // every read of this block's face table happened before the last plane's barrier
     const int nx = A.work ? (int)gridDim.x + atomicAdd(A.work, 1) : w + (int)gridDim.x;
     s_next = nx;
-    if (nx < A.nblk) {
-      const int bn = A.wl ? A.wl[nx] : nx;
+    if (nx < nitem) {
+      const int bn = A.wl ? A.wl[nx >> zs] : nx >> zs;
 #pragma unroll
       for (int f = 0; f < 6; ++f) {
         s_src[f] = A.bd[bn].src[f];

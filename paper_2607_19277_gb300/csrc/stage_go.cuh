@@ -15,18 +15,50 @@ constexpr int stage_minb() {
   return 3 * (SMEM + 1024) <= 233472 ? 3 : (2 * (SMEM + 1024) <= 233472 ? 2 : 1);
 }
 
-template <template <typename> class PT, typename R, int LIM, int FLUX, int RAW, int SFB>
+// Work items per block: a launch of few blocks is cut along z into 2^zs items of 16 >> zs planes
+// each, so that it fills the SMs (one block per CTA leaves 144 of 152 SMs idle at 8 blocks and
+// runs 16 planes in sequence). An item costs its planes and a start c (four more planes
+// loaded and converted, one more z-face) of about c = 1.1 planes in FP32 and 0.5 in FP64, whose
+// faces cost more; the SM with the most items decides, and an item alone on its SM runs slower
+// per plane than several together (by 1.4 in FP32, by 1.09 in FP64 where two CTAs fit). The
+// smallest cost by this count, whole blocks unless a cut is at least 3% better, is within 5%
+// of the fastest cut in all 13 sizes x 7 schemes timed. us per stage launch on 152 SMs, whole
+// blocks -> chosen cut: HD FP64 8 blocks 714 -> 69, 64 blocks 718 -> 356, 512 blocks 2560 ->
+// 2341; MHD FP32 8 blocks 49 -> 14, 64 blocks 50 -> 29, 210 blocks 78 -> 64, 1000 blocks 243
+// uncut (256 cut in two).
+inline int stage_zsplit(int nblk, int sms, bool fp64, int ctas_per_sm) {
+  const double c = fp64 ? 0.5 : 1.1;
+  const double lone = fp64 ? (ctas_per_sm > 1 ? 1.09 : 1.0) : 1.4;
+  int best = 0;
+  double best_cost = 0.0;
+  for (int zs = 0; zs <= 4; ++zs) {
+    const long long per_sm = (((long long)nblk << zs) + sms - 1) / sms;
+    const double cost = (double)per_sm * ((NB >> zs) + c) * (per_sm == 1 ? lone : 1.0);
+    if (zs == 0 || cost < 0.97 * best_cost) {
+      best = zs;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
+
+// Z_CUT: launches of this layout may cut blocks along z (a kernel of its own: the item bounds
+// as variables cost 1.6% on a 256^3 launch of whole blocks, 0.457 -> 0.464 ms for HD FP32).
+template <template <typename> class PT, typename R, int LIM, int FLUX, int RAW, int SFB, bool Z_CUT>
 static cudaError_t stage_go_layout(const StageArgs& a, cudaStream_t s) {
   constexpr size_t SMEM = stage_smem_bytes<PT, R, RAW, SFB>();
   constexpr int MINB = stage_minb<PT, R, RAW, SFB>();
-  auto k = stage_kernel<PT, R, LIM, FLUX, MINB, RAW, SFB>;
+  auto whole = stage_kernel<PT, R, LIM, FLUX, MINB, RAW, SFB, false>;
+  auto cut = stage_kernel<PT, R, LIM, FLUX, MINB, RAW, SFB, Z_CUT>;
   static bool attr_set = false;
   if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
+    cudaError_t e = cudaFuncSetAttribute(whole, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
+    if (e == cudaSuccess && Z_CUT)
+      e = cudaFuncSetAttribute(cut, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
-  // persistent grid: as many CTAs as fit on the GPU at once, each looping over blocks
+  // persistent grid: as many CTAs as fit on the GPU at once, each looping over work items
   static int sms = 0;
   if (!sms) {
     int dev = 0;
@@ -34,15 +66,18 @@ static cudaError_t stage_go_layout(const StageArgs& a, cudaStream_t s) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (sms <= 0) sms = 1;
   }
-  int grid = a.grid > 0 ? a.grid : MINB * sms;   // a tuned persistent grid, else the default
-  if (grid > a.nblk) grid = a.nblk;
-  if (grid <= 0) return cudaSuccess;
+  if (a.nblk <= 0) return cudaSuccess;
   StageArgs args = a;
+  args.zs = Z_CUT ? stage_zsplit(a.nblk, sms, sizeof(R) == 8, MINB) : 0;
+  int grid = a.grid > 0 ? a.grid : MINB * sms;   // a tuned persistent grid, else the default
+  if (grid > (a.nblk << args.zs)) grid = a.nblk << args.zs;
   args.ppf.set(a.gamma, 0.0);
   args.fa = (float)a.a;
   args.fb = (float)a.b;
   args.combine = a.a != 0.0 ? 1 : 0;
-  k<<<grid, 256, SMEM, s>>>(*static_cast<const CUtensorMap*>(args.tmap), args);
+  const CUtensorMap& tm = *static_cast<const CUtensorMap*>(args.tmap);
+  if (args.zs) cut<<<grid, 256, SMEM, s>>>(tm, args);
+  else whole<<<grid, 256, SMEM, s>>>(tm, args);
   return cudaGetLastError();
 }
 
@@ -53,18 +88,19 @@ static cudaError_t stage_go_layout(const StageArgs& a, cudaStream_t s) {
 // 0) takes layout 2 where it keeps as many CTAs per SM as layout 1, else layout 1 (FP32
 // stencils; FP64 keeps layout 1). Layout 3 is an autotuner choice: at equal CTAs per SM its
 // global re-read of U_s costs about what its saved barrier gains (MHD 0.870 against 0.860 ms,
-// FFHD 0.459 against 0.450 ms per 256^3 stage launch).
+// FFHD 0.459 against 0.450 ms per 256^3 stage launch). Only the default layout cuts blocks along
+// z (stage_zsplit).
 template <template <typename> class PT, typename R, int LIM, int FLUX>
 static cudaError_t stage_go(const StageArgs& a, cudaStream_t s) {
   if constexpr (sizeof(R) == 8) {
-    return stage_go_layout<PT, R, LIM, FLUX, 4, 1>(a, s);
+    return stage_go_layout<PT, R, LIM, FLUX, 4, 1, true>(a, s);
   } else {
     constexpr int dflt = stage_minb<PT, R, 5, 2>() >= stage_minb<PT, R, 4, 1>() ? STAGE_LAYOUT_RING5_DB
                                                                                  : STAGE_LAYOUT_RING4;
     const int lay = a.layout == 0 ? dflt : a.layout;
-    if (lay == STAGE_LAYOUT_RING5_DB) return stage_go_layout<PT, R, LIM, FLUX, 5, 2>(a, s);
-    if (lay == STAGE_LAYOUT_RING3_DB) return stage_go_layout<PT, R, LIM, FLUX, 3, 2>(a, s);
-    return stage_go_layout<PT, R, LIM, FLUX, 4, 1>(a, s);
+    if (lay == STAGE_LAYOUT_RING5_DB) return stage_go_layout<PT, R, LIM, FLUX, 5, 2, dflt == STAGE_LAYOUT_RING5_DB>(a, s);
+    if (lay == STAGE_LAYOUT_RING3_DB) return stage_go_layout<PT, R, LIM, FLUX, 3, 2, false>(a, s);
+    return stage_go_layout<PT, R, LIM, FLUX, 4, 1, dflt == STAGE_LAYOUT_RING4>(a, s);
   }
 }
 
