@@ -109,7 +109,7 @@ __device__ __forceinline__ void atomic_max_pos(unsigned long long* addr, double 
 }
 
 // Signal speeds of one cell, s_d = max |lambda_+-| along d, evaluated in the stencil
-// precision R (the SRHD primitive recovery inside is FP64 always); the maxima
+// precision R (the SRHD primitive recovery inside has its own precision); the maxima
 // ssum = max sum_d s_d / dx_d and smax = max_d s_d are accumulated in R (a maximum is exact
 // in any precision; the caller widens the result to FP64 once). dxr = dx rounded to R.
 template <template <typename> class PT, typename R>

@@ -1,0 +1,57 @@
+"""The FP32 stencil's relativistic recovery finishes in FP32 pairs where their guards hold, else
+in FP64. xi and Gamma of every cell of random states (read back as the auxiliaries after a step
+of negligible length, which leaves the conserved state as it is) against the root found in
+extended precision from the same FP32 conserved values: hot and cold gases, Lorentz factors up
+to 60, both equations of state, so that cells take either branch."""
+import numpy as np
+import pytest
+
+from paper_2607_19277_gb300 import agile
+
+pytestmark = pytest.mark.gpu
+
+
+def _root(cons, eos, gamma):
+    """xi, Gamma from conserved values by Newton steps in extended precision from above."""
+    L = np.longdouble
+    D, m2, E = cons[:, 0].astype(L), (cons[:, 1:4].astype(L) ** 2).sum(1), (cons[:, 4].astype(L) + cons[:, 0])
+    lo, hi = np.maximum(E, np.sqrt(m2)), (L(4) / 3 if eos == "synge" else L(gamma)) * E
+
+    def off(x):
+        w = m2 / (x * x)
+        lor = 1 / np.sqrt(1 - w)
+        rho = D / lor
+        if eos == "synge":
+            h = x / (D * lor)
+            return x - rho * (5 * h - np.sqrt(9 * h * h + 16)) / 8 - E, lor
+        return x - (L(gamma) - 1) / L(gamma) * (x * (1 - w) - rho) - E, lor
+    for _ in range(70):                       # f rises through the root: plain bisection
+        mid = (lo + hi) / 2
+        up = off(mid)[0] < 0
+        lo, hi = np.where(up, mid, lo), np.where(up, hi, mid)
+    return hi, off(hi)[1]
+
+
+@pytest.mark.parametrize("eos,gamma", [("ideal", 4.0 / 3.0), ("ideal", 5.0 / 3.0), ("synge", 4.0 / 3.0)])
+@pytest.mark.parametrize("lorentz,theta", [(1.001, (-1, 1)), (10.0, (-2, 1)), (60.0, (-1, 2)), (3.0, (-4.5, -3))])
+def test_recovery_against_extended_precision(eos, gamma, lorentz, theta):
+    rng = np.random.RandomState(11)
+    n = (2, 16, 16, 16)
+    rho = 10 ** rng.uniform(-2, 2, n)
+    u = rng.randn(3, *n)
+    u *= np.sqrt(np.exp(rng.uniform(0, np.log(lorentz), n)) ** 2 - 1) / np.sqrt((u ** 2).sum(0))
+    prim = np.stack([rho, u[0], u[1], u[2], rho * 10 ** rng.uniform(*theta, n)], axis=1)
+    m = agile.Mesh(agile.make_config(physics="srhd", limiter="minmod", flux="tvdlf", rk=2, real_bytes=4, gamma=gamma,
+                                     eos=eos, base_blocks=(2, 1, 1)))
+    m.set_state_prims(prim)
+    cons = m.get_state()[2]
+    m.step(1e-35)
+    assert np.array_equal(m.get_state()[2], cons)
+    aux = m.get_aux()
+    m.close()
+    xi, lor = _root(cons, eos, gamma)
+    # half an ulp of the FP32 result, and what the last step's first-order update leaves out:
+    # (3/2) Gamma^4 (dxi / xi)^2 of Gamma, the step dxi being at most 1e-6 xi
+    half = 2.0 ** -24 * 1.04
+    assert np.all(np.abs(aux[:, 0] / xi - 1) <= half + 2e-12)
+    assert np.all(np.abs(aux[:, 1] / lor - 1) <= half + 1.5 * lor ** 4 * 1e-12)
