@@ -341,6 +341,15 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   constexpr bool PAIRED = sizeof(R) == 4 && PairPhys<P>::OK && (FLUX == FLUX_HLL || FLUX == FLUX_TVDLF);
   constexpr int NAW = NA > 0 ? NA : 1;
   constexpr bool RESP = res_of<P>::value;   // resistive MHD sources
+  constexpr R FU = R(flux_unit<FLUX>());    // unit of the scalar solver's fluxes
+  constexpr R FUZ = PAIRED ? R(1) : FU;     // unit of the z-face fluxes
+  // FP64: the x/y slopes of a plane are formed once per cell and shared through the flux
+  // buffers (below; three more CTA barriers per plane), instead of by the faces on both sides.
+  // The FP64 units bind (86% busy at 8% of the issue slots): with the comparisons and roots
+  // taken off them (physics.cuh) this took a 96x80x112 van Leer / TVDLF HD solve from 1.17 to
+  // 0.96 ms per stage and a 128^3 MHD one from 5.5 to 4.6 ms. FP32 kernels are bound by
+  // instruction issue and barriers, and form them twice.
+  constexpr bool SHARED_SLOPES = sizeof(R) == 8;
   // A work item is planes k0 .. k0 + nz - 1 of a block (the whole block for zs = 0): it reads
   // planes k0 - 2 .. k0 + nz + 1, TMA sequence 0 .. nz + 3.
   const int zs = Z_CUT ? A.zs : 0;
@@ -606,25 +615,26 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
     if constexpr (PAIRED) riemann_z_lr<P, FLUX>(pl, pr, f, pp);
     else riemann<P, R, 2, FLUX>(pl, pr, f, pp);
   };
-  auto xface = [&](const R* C, int fi, int row, R* f) {  // x-face fi - 1/2 of row `row`
-    R a[NV], bq[NV], c[NV], d[NV], pl[NV], pr[NV];
+  // States of the face between cells q[o] and q[2 o] of a ring plane (o: the step along the
+  // face's direction), from half-slopes of the two cells in shared memory (SHARED_SLOPES) or
+  // formed here.
+  auto face_states = [&](const R* q, int o, const R* sl, const R* sr, R* pl, R* pr) {
+    if constexpr (SHARED_SLOPES) {
 #pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      const R* r = C + v * 400 + (row + 2) * 20 + fi;
-      a[v] = r[0]; bq[v] = r[1]; c[v] = r[2]; d[v] = r[3];
-    }
-    plm<NV, R, LIM, P::NREC>(a, bq, c, d, pl, pr);
-    riemann<P, R, 0, FLUX>(pl, pr, f, pp);
-  };
-  auto yface = [&](const R* C, int fj, int col, R* f) {  // y-face fj - 1/2 of column `col`
-    R a[NV], bq[NV], c[NV], d[NV], pl[NV], pr[NV];
+      for (int v = 0; v < NV; ++v) {
+        const R* r = q + v * 400;
+        pl[v] = v < P::NREC ? r[o] + sl[v * 272] : r[o];
+        pr[v] = v < P::NREC ? r[2 * o] - sr[v * 272] : r[2 * o];
+      }
+    } else {
+      R a[NV], bq[NV], c[NV], d[NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      const R* r = C + v * 400 + fj * 20 + col + 2;
-      a[v] = r[0]; bq[v] = r[20]; c[v] = r[40]; d[v] = r[60];
+      for (int v = 0; v < NV; ++v) {
+        const R* r = q + v * 400;
+        a[v] = r[0]; bq[v] = r[o]; c[v] = r[2 * o]; d[v] = r[3 * o];
+      }
+      plm<NV, R, LIM, P::NREC>(a, bq, c, d, pl, pr);
     }
-    plm<NV, R, LIM, P::NREC>(a, bq, c, d, pl, pr);
-    riemann<P, R, 1, FLUX>(pl, pr, f, pp);
   };
 
   // ---- prologue: raw planes by TMA, halo fetches of planes k0 and k0 + 1, primitives of
@@ -657,7 +667,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   zface(k0 - 1, fzd, hz);
   if (FR && k0 == 0 && slot[4] >= 0) {
 #pragma unroll
-    for (int v = 0; v < NV; ++v) FR[((size_t)slot[4] * NV + v) * 256 + cell2] = fzd[v];
+    for (int v = 0; v < NV; ++v) FR[((size_t)slot[4] * NV + v) * 256 + cell2] = FUZ * fzd[v];
   }
   convert_halo(k0);
   __syncthreads();   // plane k0 of the ring (interior and halo) is complete
@@ -789,19 +799,46 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
           }
         }
       } else {
-        xface(Ck, fc, fr, f);
+        const int xs = fr * 16 + fc, xs1 = fc < 15 ? xs + 1 : 256 + fr;   // faces of cell (fc, fr)
+        if constexpr (SHARED_SLOPES) {
+          // half-slopes of cell (fc, fr) along x and y into the slots of its upper faces; one
+          // warp adds those of the 32 halo cells -1, for the lower block-boundary faces
+          auto slope = [&](const R* q, int o) {
+            return half_slope<R, LIM>(q[o] - q[0], q[2 * o] - q[o]);
+          };
 #pragma unroll
-        for (int v = 0; v < NV; ++v) sFx[v * 272 + fr * 16 + fc] = f[v] * idx;
+          for (int v = 0; v < P::NREC; ++v) {
+            sFx[v * 272 + xs1] = slope(Ck + v * 400 + (fr + 2) * 20 + fc + 1, 1);
+            sFy[v * 272 + xs + 16] = slope(Ck + v * 400 + (fr + 1) * 20 + fc + 2, 20);
+          }
+          if (warp == 4 * (k & 1) + (((k >> 1) + 1) & 3)) {
+            const int r = t & 15;
+            const bool yd = (t & 16) != 0;
+            const R* q = Ck + (yd ? r + 2 : (r + 2) * 20);
+            R* dstp = yd ? sFy + r : sFx + r * 16;
+#pragma unroll
+            for (int v = 0; v < P::NREC; ++v) dstp[v * 272] = slope(q + v * 400, yd ? 20 : 1);
+          }
+          __syncthreads();
+        }
+        R pl[NV], pr[NV];
+        face_states(Ck + (fr + 2) * 20 + fc, 1, sFx + xs, sFx + xs1, pl, pr);
+        riemann<P, R, 0, FLUX>(pl, pr, f, pp);
+        if constexpr (SHARED_SLOPES) __syncthreads();   // every x-slope has been read
+#pragma unroll
+        for (int v = 0; v < NV; ++v) sFx[v * 272 + fr * 16 + fc] = f[v] * (FU * idx);
         if (FR && fc == 0 && slot[0] >= 0) {
 #pragma unroll
-          for (int v = 0; v < NV; ++v) FR[((size_t)slot[0] * NV + v) * 256 + k * 16 + fr] = f[v];
+          for (int v = 0; v < NV; ++v) FR[((size_t)slot[0] * NV + v) * 256 + k * 16 + fr] = FU * f[v];
         }
-        yface(Ck, fr, fc, f);
+        face_states(Ck + fr * 20 + fc + 2, 20, sFy + xs, sFy + xs + 16, pl, pr);
+        riemann<P, R, 1, FLUX>(pl, pr, f, pp);
+        if constexpr (SHARED_SLOPES) __syncthreads();   // every y-slope has been read
 #pragma unroll
-        for (int v = 0; v < NV; ++v) sFy[v * 272 + fr * 16 + fc] = f[v] * idy;
+        for (int v = 0; v < NV; ++v) sFy[v * 272 + fr * 16 + fc] = f[v] * (FU * idy);
         if (FR && fr == 0 && slot[2] >= 0) {
 #pragma unroll
-          for (int v = 0; v < NV; ++v) FR[((size_t)slot[2] * NV + v) * 256 + k * 16 + fc] = f[v];
+          for (int v = 0; v < NV; ++v) FR[((size_t)slot[2] * NV + v) * 256 + k * 16 + fc] = FU * f[v];
         }
       }
       // the 32 block-boundary faces, one warp per plane in turn, taken from the half of the
@@ -814,34 +851,49 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
         const bool yd = lane >= 16;
         const int base = yd ? 16 * 20 + r + 2 : (r + 2) * 20 + 16;
         const int stp = yd ? 20 : 1;
-        R a[NV], bq[NV], c[NV], d[NV], pl[NV], pr[NV];
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-          const R* q = Ck + v * 400 + base;
-          a[v] = q[0]; bq[v] = q[stp]; c[v] = q[2 * stp]; d[v] = q[3 * stp];
-        }
-        swap_xy<P, R>(a, yd);
-        swap_xy<P, R>(bq, yd);
-        swap_xy<P, R>(c, yd);
-        swap_xy<P, R>(d, yd);
-        plm<NV, R, LIM, P::NREC>(a, bq, c, d, pl, pr);
-        riemann<P, R, 0, FLUX>(pl, pr, f, pp);
-        swap_xy<P, R>(f, yd);
         const int fs = yd ? 1 : 0;
         R* dstp = yd ? sFy + 16 * 16 + r : sFx + 256 + r;
-        const R ids = yd ? idy : idx;
+        R pl[NV], pr[NV];
+        if constexpr (SHARED_SLOPES) {
+          // cell 15's half-slope lies in this face's slot (read by this lane only), cell 16's
+          // is formed here
+#pragma unroll
+          for (int v = 0; v < NV; ++v) {
+            const R* q = Ck + v * 400 + base;
+            const R c = q[2 * stp];
+            pl[v] = v < P::NREC ? q[stp] + dstp[v * 272] : q[stp];
+            pr[v] = v < P::NREC ? c - half_slope<R, LIM>(c - q[stp], q[3 * stp] - c) : c;
+          }
+          swap_xy<P, R>(pl, yd);
+          swap_xy<P, R>(pr, yd);
+        } else {
+          R a[NV], bq[NV], c[NV], d[NV];
+#pragma unroll
+          for (int v = 0; v < NV; ++v) {
+            const R* q = Ck + v * 400 + base;
+            a[v] = q[0]; bq[v] = q[stp]; c[v] = q[2 * stp]; d[v] = q[3 * stp];
+          }
+          swap_xy<P, R>(a, yd);
+          swap_xy<P, R>(bq, yd);
+          swap_xy<P, R>(c, yd);
+          swap_xy<P, R>(d, yd);
+          plm<NV, R, LIM, P::NREC>(a, bq, c, d, pl, pr);
+        }
+        riemann<P, R, 0, FLUX>(pl, pr, f, pp);
+        swap_xy<P, R>(f, yd);
+        const R ids = FU * (yd ? idy : idx);
 #pragma unroll
         for (int v = 0; v < NV; ++v) dstp[v * 272] = f[v] * ids;
         const int sl = slot[1 + 2 * fs];
         if (FR && sl >= 0) {
 #pragma unroll
-          for (int v = 0; v < NV; ++v) FR[((size_t)sl * NV + v) * 256 + k * 16 + r] = f[v];
+          for (int v = 0; v < NV; ++v) FR[((size_t)sl * NV + v) * 256 + k * 16 + r] = FU * f[v];
         }
       }
       zface(k, fzu, hz);
       if (FR && k == NB - 1 && slot[5] >= 0) {
 #pragma unroll
-        for (int v = 0; v < NV; ++v) FR[((size_t)slot[5] * NV + v) * 256 + cell2] = fzu[v];
+        for (int v = 0; v < NV; ++v) FR[((size_t)slot[5] * NV + v) * 256 + cell2] = FUZ * fzu[v];
       }
     }
     __syncthreads();
@@ -868,7 +920,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
         for (int v = 0; v < NV; ++v) {
           const R lx = sFx[v * 272 + fxr] - sFx[v * 272 + cell2];
           const R ly = sFy[v * 272 + (ty + 1) * 16 + tx] - sFy[v * 272 + ty * 16 + tx];
-          const R lz = (fzu[v] - fzd[v]) * idz;
+          const R lz = (fzu[v] - fzd[v]) * (FUZ * idz);
           L[v] = -((lx + ly) + lz);
           fzd[v] = fzu[v];
         }
@@ -892,7 +944,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
         for (int v = 0; v < NV; ++v) {
           const R lx = sFx[v * 272 + fxr] - sFx[v * 272 + cell2];
           const R ly = sFy[v * 272 + (ty + 1) * 16 + tx] - sFy[v * 272 + ty * 16 + tx];
-          const R lz = (fzu[v] - fzd[v]) * idz;
+          const R lz = (fzu[v] - fzd[v]) * (FUZ * idz);
           R L = -((lx + ly) + lz);
           if constexpr (RESP) {
             if (v >= P::BOFF && v < P::BOFF + 3) L = L + rsrc[v - P::BOFF];

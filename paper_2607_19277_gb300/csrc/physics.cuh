@@ -53,11 +53,42 @@ struct PhysParamsT {
 __device__ __forceinline__ float rabs(float a) { return fabsf(a); }
 __device__ __forceinline__ double rabs(double a) { return fabs(a); }
 __device__ __forceinline__ float rmin(float a, float b) { return fminf(a, b); }
-__device__ __forceinline__ double rmin(double a, double b) { return fmin(a, b); }
+// FP64 comparisons, minima and maxima run on the bit patterns: GB300 has two FP64 lanes per SM,
+// so one FP64 instruction, a comparison included, costs the issue slots of some 60 integer ones,
+// of which the FP64 stencil leaves nine tenths idle. Same results as fmin / fmax / ">": of one
+// NaN and a number the number, of two zeros -0 as the smaller. bits_key orders every value.
+__device__ __forceinline__ long long bits_key(double a) {
+  const long long i = __double_as_longlong(a);
+  return i ^ ((i >> 63) & 0x7fffffffffffffffLL);
+}
+__device__ __forceinline__ bool bits_nan(double a) {
+  return (__double_as_longlong(a) & 0x7fffffffffffffffLL) > 0x7ff0000000000000LL;
+}
+__device__ __forceinline__ bool rpos(float a) { return a > 0.0f; }
+__device__ __forceinline__ bool rpos(double a) {   // a > 0
+  return (unsigned long long)(__double_as_longlong(a) - 1) < 0x7ff0000000000000ULL;
+}
+__device__ __forceinline__ double rmin(double a, double b) {
+  return bits_nan(a) || (bits_key(b) < bits_key(a) && !bits_nan(b)) ? b : a;
+}
 __device__ __forceinline__ float rmax(float a, float b) { return fmaxf(a, b); }
-__device__ __forceinline__ double rmax(double a, double b) { return fmax(a, b); }
+__device__ __forceinline__ double rmax(double a, double b) {
+  return bits_nan(a) || (bits_key(b) > bits_key(a) && !bits_nan(b)) ? b : a;
+}
 __device__ __forceinline__ float rsqrt_(float a) { return sqrtf(a); }
-__device__ __forceinline__ double rsqrt_(double a) { return sqrt(a); }
+// FP64 square root: the hardware estimate y of a^-1/2 (PTX rsqrt.approx.ftz.f64), s = a y, and
+// with e = 1 - s y one third-order step of the series s / sqrt(1 - e) = s (1 + e/2 + 3/8 e^2),
+// whose last addition rounds once: within 1 ulp, in 5 FP64 operations (the library's root takes
+// about twice as many). Zeros, subnormal, negative and non-finite values take the library's.
+__device__ __forceinline__ double sqrt64(double a) {
+  if ((unsigned)__double2hiint(a) - 0x00100000u >= 0x7fe00000u) return sqrt(a);
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+  const double s = a * y;
+  const double e = fma(-s, y, 1.0);
+  return fma(s * e, fma(e, 0.375, 0.5), s);
+}
+__device__ __forceinline__ double rsqrt_(double a) { return sqrt64(a); }
 __device__ __forceinline__ float rsign(float a) { return copysignf(1.0f, a); }
 __device__ __forceinline__ double rsign(double a) { return copysign(1.0, a); }
 // Reciprocal and quotient in the stencil precision. FP32: the build's fast single-precision
@@ -93,11 +124,20 @@ template <> __device__ __forceinline__ double rtiny<double>() { return 1e-300; }
 template <typename R, int LIM>
 __device__ __forceinline__ R half_slope(R a, R b) {
   if (LIM == LIM_MINMOD) {
-    return (R(0.25) * (rsign(a) + rsign(b))) * rmin(rabs(a), rabs(b));
+    if constexpr (sizeof(R) == 8) {
+      // (sgn a + sgn b)/4 is +-1/2 or 0, and |a|, |b| order like their bit patterns (a NaN
+      // above every number): one FP64 operation
+      const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b);
+      const long long ma = ia & 0x7fffffffffffffffLL, mb = ib & 0x7fffffffffffffffLL;
+      const long long sg = (ia ^ ib) < 0 ? 0 : 0x3fe0000000000000LL | (ia & (long long)0x8000000000000000ULL);
+      return __longlong_as_double(sg) * __longlong_as_double(ma < mb ? ma : mb);
+    } else {
+      return (R(0.25) * (rsign(a) + rsign(b))) * rmin(rabs(a), rabs(b));
+    }
   } else {
     const R ab = a * b;
     const R q = rdiv(ab, a + b);
-    return ab > R(0) ? q : R(0);
+    return rpos(ab) ? q : R(0);
   }
 }
 
@@ -126,7 +166,7 @@ struct HdPhys {
     p[2] = vy;
     p[3] = vz;
     p[4] = g1 * (u[4] - R(0.5) * rho * (vx * vx + vy * vy + vz * vz));
-    st |= (!(rho > R(0)) | !(p[4] > R(0))) ? ST_EUNPHYS : 0;
+    st |= (!rpos(rho) | !rpos(p[4])) ? ST_EUNPHYS : 0;
   }
 
   __device__ static __forceinline__ void prim2cons(const R* p, R* u, const PhysParamsT<R>& pp) {
@@ -190,7 +230,7 @@ struct MhdPhys {
     p[6] = u[6];
     p[7] = u[7];
     p[8] = u[8];
-    st |= (!(rho > R(0)) | !(p[4] > R(0))) ? ST_EUNPHYS : 0;
+    st |= (!rpos(rho) | !rpos(p[4])) ? ST_EUNPHYS : 0;
   }
 
   __device__ static __forceinline__ void prim2cons(const R* p, R* u, const PhysParamsT<R>& pp) {
@@ -668,7 +708,7 @@ struct FfhdPhysT {
     p[2] = pp.g1 * (u[2] - R(0.5) * rho * v * v);
 #pragma unroll
     for (int i = 3; i < NV; ++i) p[i] = u[i];
-    st |= (!(rho > R(0)) | !(p[2] > R(0))) ? ST_EUNPHYS : 0;
+    st |= (!rpos(rho) | !rpos(p[2])) ? ST_EUNPHYS : 0;
   }
 
   __device__ static __forceinline__ void prim2cons(const R* p, R* u, const PhysParamsT<R>& pp) {
@@ -717,7 +757,16 @@ struct FfhdPhysT {
 template <typename R> using FfhdPhys = FfhdPhysT<R, false>;
 template <typename R> using FfhdHtcPhys = FfhdPhysT<R, true>;
 
-// Riemann flux at a face from reconstructed primitive states (modified in place).
+// The scalar solver returns the TVDLF flux times two: (F_l + F_r) - c (U_r - U_l); the halving
+// goes into the factor 1 / dx that multiplies every flux (a power of two: the same bits), which
+// takes one operation per variable and face off the FP64 units.
+template <int FLUX>
+__host__ __device__ constexpr double flux_unit() {
+  return FLUX == FLUX_TVDLF ? 0.5 : 1.0;
+}
+
+// Riemann flux at a face from reconstructed primitive states (modified in place), in units of
+// flux_unit<FLUX>().
 template <class P, typename R, int D, int FLUX>
 __device__ __forceinline__ void riemann(R* pl, R* pr, R* f, const PhysParamsT<R>& pp) {
   constexpr int NV = P::NV;
@@ -762,9 +811,9 @@ __device__ __forceinline__ void riemann(R* pl, R* pr, R* f, const PhysParamsT<R>
     const R c = rmax(rmax(rabs(lml), rabs(lpl)), rmax(rabs(lmr), rabs(lpr)));
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-      if (v >= P::FROZEN) f[v] = fl[v];   // frozen variables: exact flux, no dissipation
-      else if (v == P::QV) f[v] = R(0);   // no flux term at all
-      else f[v] = R(0.5) * (fl[v] + fr[v]) - R(0.5) * c * (ur[v] - ul[v]);
+      if (v >= P::FROZEN) f[v] = fl[v] + fl[v];   // frozen variables: exact flux, no dissipation
+      else if (v == P::QV) f[v] = R(0);           // no flux term at all
+      else f[v] = (fl[v] + fr[v]) - c * (ur[v] - ul[v]);
     }
   } else {
     const R sl = rmin(rmin(lml, lmr), R(0));
