@@ -303,12 +303,21 @@ __device__ __forceinline__ int pslot(int p) { return (p + 3) % 3; }
 template <template <typename> class PT, typename R, int RAW, int SFB>
 struct StageSmem {
   static constexpr int NV = PT<R>::NV, NT = PT<R>::NV + PT<R>::NA;
+  // x-face fluxes: row r, faces 0 .. 16; y-face fluxes: faces 0 .. 16, column c. FP32 rows are 20
+  // wide, so that a warp's two rows (r, r + 4) lie 16 banks apart; FP64 rows (a half-warp covers
+  // the banks) 16, the last x-face of each row after the others.
+  static constexpr int FP = sizeof(R) == 4 ? 20 : 16;
+  static constexpr int FXN = sizeof(R) == 4 ? 16 * 20 : 272;
+  static constexpr int FYN = sizeof(R) == 4 ? 16 * 20 + 16 : 272;
+  __host__ __device__ static constexpr int xf(int r, int f) {
+    return sizeof(R) == 4 || f < 16 ? r * FP + f : 256 + r;
+  }
   static constexpr size_t bars = 128;                                  // RAW mbarriers (+pad)
   static constexpr size_t raw = bars;                                  // [RAW][NT][256]
   static constexpr size_t ring = raw + sizeof(R) * RAW * NT * 256;     // [3][NT][20 x 20]
-  static constexpr size_t fx = ring + sizeof(R) * 3 * NT * 400;        // [SFB][NV][16 x 16 + 16]
-  static constexpr size_t fy = fx + sizeof(R) * SFB * NV * 272;        // [SFB][NV][17][16]
-  static constexpr size_t total = fy + sizeof(R) * SFB * NV * 272;
+  static constexpr size_t fx = ring + sizeof(R) * 3 * NT * 400;        // [SFB][NV][FXN]
+  static constexpr size_t fy = fx + sizeof(R) * SFB * NV * FXN;        // [SFB][NV][FYN]
+  static constexpr size_t total = fy + sizeof(R) * SFB * NV * FYN;
 };
 
 // The per-stage macro-kernel. Plane k of a block is one iteration:
@@ -374,17 +383,20 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   const R* __restrict__ Rg = PRIMIN ? static_cast<const R*>(A.WG) : G;
 
   const int t = threadIdx.x;
-  const int tx = t & 15, ty = t >> 4;
   const int warp = t >> 5;
+  // Column and row of this thread's cell, which is also the cell whose lower x- and y-face it
+  // solves: the two half-warps of warp w on rows (w & 3) + 8 (w >> 2) and 4 rows further, which
+  // rows 20 wide put 16 banks apart (FP32: ring planes and flux buffers without bank conflicts;
+  // the raw planes, 16 wide as the TMA writes them, take two passes). With rows 2 w and 2 w + 1
+  // for the cell, as the raw planes prefer, each access of the ring and of the fluxes took two:
+  // 256^3 launches HD 445 -> 441 us, MHD 869 -> 862, 420 blocks FFHD with conduction 75 -> 71.
+  const int tx = t & 15, ty = (warp & 3) + 8 * (warp >> 2) + 4 * ((t >> 4) & 1);
   const int cell2 = ty * 16 + tx;
   const int cellp = (ty + 2) * 20 + tx + 2;   // this thread's cell in a 20 x 20 ring plane
-  // Faces of the x/y pass: column fc of row fr, the two half-warps of warp w on rows
-  // (w & 3) + 8 (w >> 2) and 4 rows further, which the 20-wide plane rows put 16 banks apart
-  // (the four-cell stencil loads are free of bank conflicts).
-  const int fc = tx;
-  const int fr = (warp & 3) + 8 * (warp >> 2) + 4 * ((t >> 4) & 1);
-  // x-face fluxes: [NV][16 rows][16] for faces 0..15 of each row, then [NV][16] for face 16
-  const int fxr = tx < 15 ? cell2 + 1 : 256 + ty;   // this cell's right x-face
+  // slots of its lower and upper x- and y-face in the flux buffers
+  constexpr int FP = S::FP, FXN = S::FXN, FYN = S::FYN;
+  const int fx0 = S::xf(ty, tx), fx1 = S::xf(ty, tx + 1);
+  const int fy0 = ty * FP + tx, fy1 = fy0 + FP;
   // Halo cell of this thread: h < 64 x-faces, above y-faces; the half t >> 7 of the CTA owns
   // the halo of the planes of its parity.
   const int hh = t & 127;
@@ -616,15 +628,16 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
     else riemann<P, R, 2, FLUX>(pl, pr, f, pp);
   };
   // States of the face between cells q[o] and q[2 o] of a ring plane (o: the step along the
-  // face's direction), from half-slopes of the two cells in shared memory (SHARED_SLOPES) or
+  // face's direction), from half-slopes of the two cells in shared memory (SHARED_SLOPES; ns
+  // apart per variable) or
   // formed here.
-  auto face_states = [&](const R* q, int o, const R* sl, const R* sr, R* pl, R* pr) {
+  auto face_states = [&](const R* q, int o, const R* sl, const R* sr, int ns, R* pl, R* pr) {
     if constexpr (SHARED_SLOPES) {
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         const R* r = q + v * 400;
-        pl[v] = v < P::NREC ? r[o] + sl[v * 272] : r[o];
-        pr[v] = v < P::NREC ? r[2 * o] - sr[v * 272] : r[2 * o];
+        pl[v] = v < P::NREC ? r[o] + sl[v * ns] : r[o];
+        pr[v] = v < P::NREC ? r[2 * o] - sr[v * ns] : r[2 * o];
       }
     } else {
       R a[NV], bq[NV], c[NV], d[NV];
@@ -682,8 +695,8 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   R Tkm1 = R(0);   // conduction: T = p / rho of this column at plane k - 1
   R Bkm1[3] = {R(0), R(0), R(0)};   // resistivity: B of this column at plane k - 1
   for (int k = k0; k < k1; ++k) {
-    R* sFx = sFx0 + (SFB == 2 ? (k & 1) : 0) * NV * 272;
-    R* sFy = sFy0 + (SFB == 2 ? (k & 1) : 0) * NV * 272;
+    R* sFx = sFx0 + (SFB == 2 ? (k & 1) : 0) * NV * FXN;
+    R* sFy = sFy0 + (SFB == 2 ? (k & 1) : 0) * NV * FYN;
     if (RAW == 4 && t == 0 && k > k0 && k + 3 <= k1 + 1) {
       fence_proxy_async();
       issue(k + 3);   // raw slot of plane k-1, read by its update before the previous barrier
@@ -758,13 +771,13 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
     {
       R f[NV];
       if constexpr (PAIRED) {
-        // the x-face fc - 1/2 of row fr and the y-face fr - 1/2 of column fc as one pair, the
+        // the lower x-face and the lower y-face of cell (tx, ty) as one pair, the
         // y-face's states with x and y components exchanged
         f2 a[NV], bq[NV], c[NV], d[NV], pl[NV], pr[NV], fp[NV];
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
-          const R* rx = Ck + v * 400 + (fr + 2) * 20 + fc;
-          const R* ry = Ck + swapv<P>(v) * 400 + fr * 20 + fc + 2;
+          const R* rx = Ck + v * 400 + (ty + 2) * 20 + tx;
+          const R* ry = Ck + swapv<P>(v) * 400 + ty * 20 + tx + 2;
           a[v] = f2_of(rx[0], ry[0]);
           bq[v] = f2_of(rx[1], ry[20]);
           c[v] = f2_of(rx[2], ry[40]);
@@ -779,66 +792,66 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
         for (int v = 0; v < NV; ++v) {
           R sx, sy;
           f2_split(fp[v] * kxy, sx, sy);
-          sFx[v * 272 + fr * 16 + fc] = sx;
-          sFy[swapv<P>(v) * 272 + fr * 16 + fc] = sy;
+          sFx[v * FXN + fx0] = sx;
+          sFy[swapv<P>(v) * FYN + fy0] = sy;
         }
-        if (FR && fc == 0 && slot[0] >= 0) {
+        if (FR && tx == 0 && slot[0] >= 0) {
 #pragma unroll
           for (int v = 0; v < NV; ++v) {
             R fx_, fy_;
             f2_split(fp[v], fx_, fy_);
-            FR[((size_t)slot[0] * NV + v) * 256 + k * 16 + fr] = fx_;
+            FR[((size_t)slot[0] * NV + v) * 256 + k * 16 + ty] = fx_;
           }
         }
-        if (FR && fr == 0 && slot[2] >= 0) {
+        if (FR && ty == 0 && slot[2] >= 0) {
 #pragma unroll
           for (int v = 0; v < NV; ++v) {
             R fx_, fy_;
             f2_split(fp[v], fx_, fy_);
-            FR[((size_t)slot[2] * NV + swapv<P>(v)) * 256 + k * 16 + fc] = fy_;
+            FR[((size_t)slot[2] * NV + swapv<P>(v)) * 256 + k * 16 + tx] = fy_;
           }
         }
       } else {
-        const int xs = fr * 16 + fc, xs1 = fc < 15 ? xs + 1 : 256 + fr;   // faces of cell (fc, fr)
         if constexpr (SHARED_SLOPES) {
-          // half-slopes of cell (fc, fr) along x and y into the slots of its upper faces; one
+          // half-slopes of cell (tx, ty) along x and y into the slots of its upper faces; one
           // warp adds those of the 32 halo cells -1, for the lower block-boundary faces
           auto slope = [&](const R* q, int o) {
             return half_slope<R, LIM>(q[o] - q[0], q[2 * o] - q[o]);
           };
 #pragma unroll
           for (int v = 0; v < P::NREC; ++v) {
-            sFx[v * 272 + xs1] = slope(Ck + v * 400 + (fr + 2) * 20 + fc + 1, 1);
-            sFy[v * 272 + xs + 16] = slope(Ck + v * 400 + (fr + 1) * 20 + fc + 2, 20);
+            sFx[v * FXN + fx1] = slope(Ck + v * 400 + (ty + 2) * 20 + tx + 1, 1);
+            sFy[v * FYN + fy1] = slope(Ck + v * 400 + (ty + 1) * 20 + tx + 2, 20);
           }
           if (warp == 4 * (k & 1) + (((k >> 1) + 1) & 3)) {
             const int r = t & 15;
             const bool yd = (t & 16) != 0;
             const R* q = Ck + (yd ? r + 2 : (r + 2) * 20);
-            R* dstp = yd ? sFy + r : sFx + r * 16;
+            R* dstp = yd ? sFy + r : sFx + S::xf(r, 0);
+            const int ns = yd ? FYN : FXN;
 #pragma unroll
-            for (int v = 0; v < P::NREC; ++v) dstp[v * 272] = slope(q + v * 400, yd ? 20 : 1);
+            for (int v = 0; v < P::NREC; ++v) dstp[v * ns] = slope(q + v * 400, yd ? 20 : 1);
           }
           __syncthreads();
         }
         R pl[NV], pr[NV];
-        face_states(Ck + (fr + 2) * 20 + fc, 1, sFx + xs, sFx + xs1, pl, pr);
+        face_states(Ck + (ty + 2) * 20 + tx, 1, sFx + fx0, sFx + fx1, FXN, pl, pr);
         riemann<P, R, 0, FLUX>(pl, pr, f, pp);
         if constexpr (SHARED_SLOPES) __syncthreads();   // every x-slope has been read
 #pragma unroll
-        for (int v = 0; v < NV; ++v) sFx[v * 272 + fr * 16 + fc] = f[v] * (FU * idx);
-        if (FR && fc == 0 && slot[0] >= 0) {
+        for (int v = 0; v < NV; ++v) sFx[v * FXN + fx0] = f[v] * (FU * idx);
+        if (FR && tx == 0 && slot[0] >= 0) {
 #pragma unroll
-          for (int v = 0; v < NV; ++v) FR[((size_t)slot[0] * NV + v) * 256 + k * 16 + fr] = FU * f[v];
+          for (int v = 0; v < NV; ++v) FR[((size_t)slot[0] * NV + v) * 256 + k * 16 + ty] = FU * f[v];
         }
-        face_states(Ck + fr * 20 + fc + 2, 20, sFy + xs, sFy + xs + 16, pl, pr);
+        face_states(Ck + ty * 20 + tx + 2, 20, sFy + fy0, sFy + fy1, FYN, pl, pr);
         riemann<P, R, 1, FLUX>(pl, pr, f, pp);
         if constexpr (SHARED_SLOPES) __syncthreads();   // every y-slope has been read
 #pragma unroll
-        for (int v = 0; v < NV; ++v) sFy[v * 272 + fr * 16 + fc] = f[v] * (FU * idy);
-        if (FR && fr == 0 && slot[2] >= 0) {
+        for (int v = 0; v < NV; ++v) sFy[v * FYN + fy0] = f[v] * (FU * idy);
+        if (FR && ty == 0 && slot[2] >= 0) {
 #pragma unroll
-          for (int v = 0; v < NV; ++v) FR[((size_t)slot[2] * NV + v) * 256 + k * 16 + fc] = FU * f[v];
+          for (int v = 0; v < NV; ++v) FR[((size_t)slot[2] * NV + v) * 256 + k * 16 + tx] = FU * f[v];
         }
       }
       // the 32 block-boundary faces, one warp per plane in turn, taken from the half of the
@@ -852,7 +865,8 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
         const int base = yd ? 16 * 20 + r + 2 : (r + 2) * 20 + 16;
         const int stp = yd ? 20 : 1;
         const int fs = yd ? 1 : 0;
-        R* dstp = yd ? sFy + 16 * 16 + r : sFx + 256 + r;
+        R* dstp = yd ? sFy + 16 * FP + r : sFx + S::xf(r, 16);
+        const int ns = yd ? FYN : FXN;
         R pl[NV], pr[NV];
         if constexpr (SHARED_SLOPES) {
           // cell 15's half-slope lies in this face's slot (read by this lane only), cell 16's
@@ -861,7 +875,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
           for (int v = 0; v < NV; ++v) {
             const R* q = Ck + v * 400 + base;
             const R c = q[2 * stp];
-            pl[v] = v < P::NREC ? q[stp] + dstp[v * 272] : q[stp];
+            pl[v] = v < P::NREC ? q[stp] + dstp[v * ns] : q[stp];
             pr[v] = v < P::NREC ? c - half_slope<R, LIM>(c - q[stp], q[3 * stp] - c) : c;
           }
           swap_xy<P, R>(pl, yd);
@@ -883,7 +897,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
         swap_xy<P, R>(f, yd);
         const R ids = FU * (yd ? idy : idx);
 #pragma unroll
-        for (int v = 0; v < NV; ++v) dstp[v * 272] = f[v] * ids;
+        for (int v = 0; v < NV; ++v) dstp[v * ns] = f[v] * ids;
         const int sl = slot[1 + 2 * fs];
         if (FR && sl >= 0) {
 #pragma unroll
@@ -918,8 +932,8 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
         R L[NV];
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
-          const R lx = sFx[v * 272 + fxr] - sFx[v * 272 + cell2];
-          const R ly = sFy[v * 272 + (ty + 1) * 16 + tx] - sFy[v * 272 + ty * 16 + tx];
+          const R lx = sFx[v * FXN + fx1] - sFx[v * FXN + fx0];
+          const R ly = sFy[v * FYN + fy1] - sFy[v * FYN + fy0];
           const R lz = (fzu[v] - fzd[v]) * (FUZ * idz);
           L[v] = -((lx + ly) + lz);
           fzd[v] = fzu[v];
@@ -942,8 +956,8 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
       } else {
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
-          const R lx = sFx[v * 272 + fxr] - sFx[v * 272 + cell2];
-          const R ly = sFy[v * 272 + (ty + 1) * 16 + tx] - sFy[v * 272 + ty * 16 + tx];
+          const R lx = sFx[v * FXN + fx1] - sFx[v * FXN + fx0];
+          const R ly = sFy[v * FYN + fy1] - sFy[v * FYN + fy0];
           const R lz = (fzu[v] - fzd[v]) * (FUZ * idz);
           R L = -((lx + ly) + lz);
           if constexpr (RESP) {

@@ -266,6 +266,12 @@ struct PairPhys<FfhdPhysT<float, HTC>> {
   }
 };
 
+// B_x and psi of GLM-MHD: both face states carry the same values and flux, which is the face's.
+template <class P>
+__host__ __device__ constexpr bool glm_var(int v) {
+  return P::GLM && (v == P::BOFF || v == P::NV - 1);
+}
+
 // HLL or TVDLF flux of the pair from reconstructed primitive states (modified in place).
 template <class P, int FLUX>
 __device__ __forceinline__ void riemann2(f2* pl, f2* pr, f2* f, const PairK& k) {
@@ -287,15 +293,19 @@ __device__ __forceinline__ void riemann2(f2* pl, f2* pr, f2* f, const PairK& k) 
     for (int v = 0; v < NV; ++v) {
       if (v >= P::FROZEN) f[v] = fl[v];   // frozen variables: exact flux, no dissipation
       else if (v == P::QV) f[v] = k.zero; // no flux term at all
+      else if (glm_var<P>(v)) f[v] = fl[v];
       else f[v] = fma2(nhc, ur[v] - ul[v], k.half * (fl[v] + fr[v]));
     }
   } else {
     const f2 sl = min2(min2(lml, lmr), k.zero);
     const f2 sr = max2(max2(lpl, lpr), k.zero);
     const f2 inv = rcp2(sr - sl);
-    const f2 wl = sr * inv, nwr = (k.zero - sl) * inv, wd = sl * sr * inv;
+    const f2 wl = sr * inv, nwr = (k.zero - sl) * inv, wd = sl * wl;
 #pragma unroll
-    for (int v = 0; v < NV; ++v) f[v] = fma2(wd, ur[v] - ul[v], fma2(wl, fl[v], nwr * fr[v]));
+    for (int v = 0; v < NV; ++v) {
+      if (glm_var<P>(v)) f[v] = fl[v];
+      else f[v] = fma2(wd, ur[v] - ul[v], fma2(wl, fl[v], nwr * fr[v]));
+    }
   }
 }
 
@@ -328,14 +338,17 @@ __device__ __forceinline__ void riemann_z_lr(float* pl, float* pr, float* f, con
     const float sl = fminf(fminf(lml, lmr), 0.0f);
     const float sr = fmaxf(fmaxf(lpl, lpr), 0.0f);
     const float inv = 1.0f / (sr - sl);
-    const float wd = sl * sr * inv;
-    w = f2_of(sr * inv, -(sl * inv));
+    const float wl = sr * inv, wd = sl * wl;
+    w = f2_of(wl, -(sl * inv));
     dw = f2_of(-wd, wd);
   }
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
     float a, b;
     if (FLUX == FLUX_TVDLF && v >= P::FROZEN) {          // frozen: the left flux exactly
+      f2_split(fq[v], a, b);
+      f[Q::zrot(v)] = a;
+    } else if (glm_var<P>(v)) {                          // rotated: B_z and psi
       f2_split(fq[v], a, b);
       f[Q::zrot(v)] = a;
     } else if (FLUX == FLUX_TVDLF && v == P::QV) {       // no flux term
