@@ -36,7 +36,7 @@ struct BlockDesc {
   int nbr[NFACE][4];    // finer: the 4 fine blocks (t1 + 2 t2); coarser: [0] = coarse block
   double dx[3];
   int level;
-  int pad;
+  int corrected;        // a face of the block takes the flux correction (a finer neighbour)
 };
 
 struct GhostTask {      // one coarse-fine face of a block, filled before each stage

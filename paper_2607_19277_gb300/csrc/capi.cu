@@ -41,6 +41,7 @@ struct agile_mesh {
   int* d_wl = nullptr;             // stage kernel work order (blocks by level, z-slab, 2-D Morton)
   GhostTask* d_ghosts = nullptr;
   FixupTask* d_fix = nullptr;
+  int* d_fixblk = nullptr;          // the blocks with corrected faces (one per fix-up task)
   int nghost = 0, nfix = 0;
   int* d_status = nullptr;
   unsigned long long* d_speeds = nullptr;
@@ -297,6 +298,7 @@ agile_status rebuild(agile_mesh* m) {
   dfree_t(m, m->d_bd);
   dfree_t(m, m->d_ghosts);
   dfree_t(m, m->d_fix);
+  dfree_t(m, m->d_fixblk);
   dfree(m, m->G);
   dfree(m, m->FR);
   dfree(m, m->U[1]);
@@ -315,11 +317,14 @@ agile_status rebuild(agile_mesh* m) {
   m->d_bd = (BlockDesc*)dalloc(m, desc.size() * sizeof(BlockDesc));
   m->d_ghosts = (GhostTask*)dalloc(m, ghosts.size() * sizeof(GhostTask));
   m->d_fix = (FixupTask*)dalloc(m, fix.size() * sizeof(FixupTask));
+  std::vector<int> fixblk;
+  for (const FixupTask& t : fix) fixblk.push_back(t.blk);
+  m->d_fixblk = (int*)dalloc(m, fixblk.size() * sizeof(int));
   m->G = dalloc(m, (size_t)nslots * m->nt * 512 * m->rb);
   m->FR = dalloc(m, (size_t)nslots * m->nv * 256 * m->rb);
   m->U[1] = dalloc(m, pool_bytes(m, m->nblk));
   m->U[2] = m->cfg.rk == 3 ? dalloc(m, pool_bytes(m, m->nblk)) : nullptr;
-  if (!m->d_bd || !m->d_wl || !m->d_ghosts || !m->d_fix || !m->G || !m->FR || !m->U[1] ||
+  if (!m->d_bd || !m->d_wl || !m->d_ghosts || !m->d_fix || !m->d_fixblk || !m->G || !m->FR || !m->U[1] ||
       (m->cfg.rk == 3 && !m->U[2]))
     return fail(m, AGILE_ENOMEM, "device allocation failed");
   CK(m, cudaMemcpyAsync(m->d_bd, desc.data(), desc.size() * sizeof(BlockDesc), cudaMemcpyHostToDevice, m->stream));
@@ -327,8 +332,10 @@ agile_status rebuild(agile_mesh* m) {
     CK(m, cudaMemcpyAsync(m->d_wl, order.data(), order.size() * sizeof(int), cudaMemcpyHostToDevice, m->stream));
   if (!ghosts.empty())
     CK(m, cudaMemcpyAsync(m->d_ghosts, ghosts.data(), ghosts.size() * sizeof(GhostTask), cudaMemcpyHostToDevice, m->stream));
-  if (!fix.empty())
+  if (!fix.empty()) {
     CK(m, cudaMemcpyAsync(m->d_fix, fix.data(), fix.size() * sizeof(FixupTask), cudaMemcpyHostToDevice, m->stream));
+    CK(m, cudaMemcpyAsync(m->d_fixblk, fixblk.data(), fixblk.size() * sizeof(int), cudaMemcpyHostToDevice, m->stream));
+  }
   m->nghost = (int)ghosts.size();
   m->nfix = (int)fix.size();
   m->nslots = nslots;
@@ -604,6 +611,7 @@ void agile_mesh_destroy(agile_mesh* m) {
   dfree(m, m->WG);
   dfree_t(m, m->d_ghosts);
   dfree_t(m, m->d_fix);
+  dfree_t(m, m->d_fixblk);
   dfree_t(m, m->d_status);
   dfree_t(m, m->d_speeds);
   dfree_t(m, m->d_dtch);
@@ -717,9 +725,11 @@ agile_status agile_step(agile_mesh* m, double dt) {
   static const double w2[2][2] = {{0.0, 1.0}, {0.5, 0.5}};
   static const double w3[3][2] = {{0.0, 1.0}, {0.75, 0.25}, {1.0 / 3.0, 2.0 / 3.0}};
   const int nst = m->cfg.rk;
-  const bool fuse = m->nfix == 0;
+  // the last stage applies the second GLM half and reduces the CFL maxima of U^{n+1} as it stores
+  // (maxima: unless losses follow, or the next step's first pass has them); blocks with
+  // corrected faces, a small part of a refined mesh, are left to a pass over them after the fix-up
   const bool cool = m->cool.nseg > 0;
-  const bool speeds_in_stage = fuse && !cool && !lead;   // else the post-step pass reduces them
+  const bool speeds_in_stage = !cool && !lead;
   if (cool) {                                   // first Strang half of the losses
     AuxArgs a = aux_args(m, m->U[0]);
     CK(m, launch_cooling(a, m->cool, m->d_cool, m->d_dtch, 0.5, nullptr, m->stream));
@@ -746,7 +756,7 @@ agile_status agile_step(agile_mesh* m, double dt) {
     A.glm_alpha = m->cfg.glm_alpha;
     A.htc_kappa0 = m->cfg.htc_kappa0;
     A.eta = m->cfg.eta;
-    A.glm_post = (mhd && last && fuse) ? 1 : 0;
+    A.glm_post = (mhd && last) ? 1 : 0;
     A.nblk = m->nblk;
     A.wl = m->d_wl;
     A.status = m->d_status;
@@ -790,10 +800,18 @@ agile_status agile_step(agile_mesh* m, double dt) {
       m->total_launches++;
     }
   }
-  if (mhd && !fuse) {
+  if (m->nfix && (mhd || speeds_in_stage)) {    // what the last stage left out
     AuxArgs a = aux_args(m, m->U[0]);
-    CK(m, launch_glm_decay(a, m->d_dtch, m->stream));
-    m->total_launches++;
+    a.wl = m->d_fixblk;
+    a.nblk = m->nfix;
+    if (mhd) {
+      CK(m, launch_glm_decay(a, m->d_dtch, m->stream));
+      m->total_launches++;
+    }
+    if (speeds_in_stage) {
+      CK(m, launch_speeds(a, m->d_speeds, m->stream));
+      m->total_launches++;
+    }
   }
   if (cool) {                                   // second half, with the CFL speeds of U^{n+1}
     CK(m, cudaMemsetAsync(m->d_speeds, 0, 2 * sizeof(unsigned long long), m->stream));
@@ -801,14 +819,8 @@ agile_status agile_step(agile_mesh* m, double dt) {
     CK(m, launch_cooling(a, m->cool, m->d_cool, m->d_dtch, 0.5, m->d_speeds, m->stream));
     m->total_launches++;
     m->speeds_valid = true;
-  } else if (lead) {
-    m->speeds_valid = false;                   // the next step's first pass reduces them
-  } else if (fuse) {
-    m->speeds_valid = true;
   } else {
-    m->speeds_valid = false;
-    s = ensure_speeds(m);
-    if (s) return s;
+    m->speeds_valid = !lead;                   // lead: the next step's first pass reduces them
   }
   return AGILE_OK;
 }
@@ -1172,6 +1184,7 @@ struct agile_batch {
   void* FR = nullptr;
   GhostTask* d_ghosts = nullptr;
   FixupTask* d_fix = nullptr;
+  int* d_fixblk = nullptr;          // the blocks with corrected faces (one per fix-up task)
   int nghost = 0, nfix = 0, nslots = 0;
   std::vector<agile_ic_fn> ics;     // initial conditions, re-applied to blocks a regrid creates
   std::vector<void*> ic_users;
@@ -1522,6 +1535,7 @@ agile_status batch_rebuild(agile_batch* B) {
   dfree_t(&view, B->d_wl);
   dfree_t(&view, B->d_ghosts);
   dfree_t(&view, B->d_fix);
+  dfree_t(&view, B->d_fixblk);
   dfree(&view, B->G);
   dfree(&view, B->FR);
   const bool prim_pass = phys_prim_pass(phys_kind(B->cfg));
@@ -1554,13 +1568,18 @@ agile_status batch_rebuild(agile_batch* B) {
     B->d_wl = (int*)dalloc(&view, (size_t)B->cap * sizeof(int));
   }
   if (!ghosts.empty()) B->d_ghosts = (GhostTask*)dalloc(&view, ghosts.size() * sizeof(GhostTask));
-  if (!fix.empty()) B->d_fix = (FixupTask*)dalloc(&view, fix.size() * sizeof(FixupTask));
+  std::vector<int> fixblk;
+  for (const FixupTask& t : fix) fixblk.push_back(t.blk);
+  if (!fix.empty()) {
+    B->d_fix = (FixupTask*)dalloc(&view, fix.size() * sizeof(FixupTask));
+    B->d_fixblk = (int*)dalloc(&view, fixblk.size() * sizeof(int));
+  }
   if (slots) {
     B->G = dalloc(&view, (size_t)slots * B->nt * 512 * B->rb);
     B->FR = dalloc(&view, (size_t)slots * B->nv * 256 * B->rb);
   }
   if ((B->cap && (!B->d_bd || !B->d_solve_of || !B->d_wl)) || (!ghosts.empty() && !B->d_ghosts) ||
-      (!fix.empty() && !B->d_fix) || (slots && (!B->G || !B->FR)))
+      (!fix.empty() && (!B->d_fix || !B->d_fixblk)) || (slots && (!B->G || !B->FR)))
     return bfail(B, AGILE_ENOMEM, "device allocation failed");
   B->tab_cap = B->cap;
   if (extent) {
@@ -1572,8 +1591,10 @@ agile_status batch_rebuild(agile_batch* B) {
     BCK(B, cudaMemcpyAsync(B->d_wl, work.data(), work.size() * sizeof(int), cudaMemcpyHostToDevice, B->stream));
   if (!ghosts.empty())
     BCK(B, cudaMemcpyAsync(B->d_ghosts, ghosts.data(), ghosts.size() * sizeof(GhostTask), cudaMemcpyHostToDevice, B->stream));
-  if (!fix.empty())
+  if (!fix.empty()) {
     BCK(B, cudaMemcpyAsync(B->d_fix, fix.data(), fix.size() * sizeof(FixupTask), cudaMemcpyHostToDevice, B->stream));
+    BCK(B, cudaMemcpyAsync(B->d_fixblk, fixblk.data(), fixblk.size() * sizeof(int), cudaMemcpyHostToDevice, B->stream));
+  }
   // (pageable host sources are staged when each copy is enqueued: the vectors may go now)
   B->nghost = (int)ghosts.size();
   B->nfix = (int)fix.size();
@@ -1780,7 +1801,6 @@ agile_status batch_enqueue_step(agile_batch* B) {
   static const double w2[2][2] = {{0.0, 1.0}, {0.5, 0.5}};
   static const double w3[3][2] = {{0.0, 1.0}, {0.75, 0.25}, {1.0 / 3.0, 2.0 / 3.0}};
   const int nst = B->cfg.rk;
-  const bool fuse = B->nfix == 0;     // no flux fix-up: GLM half and CFL speeds in the last stage
   for (int st = 0; st < nst; ++st) {
     const bool last = st == nst - 1;
     void* Us = st == 0 ? B->U[0] : B->U[st];
@@ -1802,11 +1822,11 @@ agile_status batch_enqueue_step(agile_batch* B) {
     A.gamma = B->cfg.gamma;
     A.glm_alpha = B->cfg.glm_alpha;
     A.htc_kappa0 = B->cfg.htc_kappa0;
-    A.glm_post = (mhd && last && fuse) ? 1 : 0;
+    A.glm_post = (mhd && last) ? 1 : 0;
     A.nblk = B->nwork;
     A.wl = B->d_wl;
     A.status = B->d_status;
-    A.speeds = (last && fuse && !lead) ? B->d_speeds : nullptr;
+    A.speeds = (last && !lead) ? B->d_speeds : nullptr;
     A.tmap = &B->tmap[st == 0 ? 0 : st];
     A.solve_of = B->d_solve_of;
     A.work = B->dynamic ? B->d_work + st : nullptr;
@@ -1836,8 +1856,10 @@ agile_status batch_enqueue_step(agile_batch* B) {
       BCK(B, launch_fixup(fa, B->d_fix, B->nfix, A.b, B->d_dtch, B->stream));
     }
   }
-  if (!fuse) {                        // after the last fix-up: GLM half, then the CFL speeds
+  if (B->nfix) {                      // after the last fix-up: GLM half and CFL maxima of its blocks
     AuxArgs a = batch_aux(B, B->U[0]);
+    a.wl = B->d_fixblk;
+    a.nblk = B->nfix;
     if (mhd) BCK(B, launch_glm_decay(a, B->d_dtch, B->stream));
     if (!lead) BCK(B, launch_speeds(a, B->d_speeds, B->stream));
   }
@@ -2077,6 +2099,7 @@ void agile_batch_destroy(agile_batch* B) {
   dfree_t(&view, B->d_wl);
   dfree_t(&view, B->d_ghosts);
   dfree_t(&view, B->d_fix);
+  dfree_t(&view, B->d_fixblk);
   dfree(&view, B->G);
   dfree(&view, B->FR);
   dfree(&view, B->W);

@@ -32,10 +32,12 @@ struct StageArgs {
   double a, b;              // U_out = a U^n + b (U_s + dt L(U_s))
   double gamma;
   double glm_alpha;
-  int glm_post;             // multiply psi of the output by exp(-dt/2 c_h alpha / min dx)
+  int glm_post;             // multiply psi of the output by exp(-dt/2 c_h alpha / min dx) (not on
+                            // blocks with corrected faces)
   int nblk;
   int* status;
-  unsigned long long* speeds;   // fused reduction of [max sum_d s_d/dx_d, max s_d] per solve, or nullptr
+  unsigned long long* speeds;   // fused reduction of [max sum_d s_d/dx_d, max s_d] per solve over the
+                                // blocks without corrected faces, or nullptr
   const void* tmap;             // host CUtensorMap of the pool Us, or of W for a physics with a
                                 // primitive-recovery pass (x, y, z, block*var)
   const void* W = nullptr;      // primitives (and auxiliaries) of Us, per block as Us, from the
@@ -460,8 +462,10 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   const int b = A.wl ? A.wl[w >> zs] : w >> zs;
   const int k0 = (w & ((1 << zs) - 1)) * nz, k1 = k0 + nz;
   const int sv = A.solve_of ? A.solve_of[b] : 0;
-  unsigned long long* speeds = A.speeds ? A.speeds + 2 * sv : nullptr;
   const BlockDesc& bd = A.bd[b];
+  // a block whose faces are corrected after this launch gets its CFL maxima and the second GLM
+  // half after that
+  unsigned long long* speeds = A.speeds && !bd.corrected ? A.speeds + 2 * sv : nullptr;
   if (sv != key_sv || bd.level != key_lev) {   // CTA-uniform: every thread takes it or none
     // one thread forms the constants in FP64 (divisions, the exp) and the CTA reads them
     // back, so the FP64 units see one thread's work per change instead of the CTA's
@@ -503,6 +507,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
     key_lev = bd.level;
   }
 
+  const R psi_post = bd.corrected ? R(1) : glm_fr;   // second GLM half of psi
   // plane p (k0 - 2 .. k1 + 1) -> TMA sequence q = p - k0 + 2, raw slot q % RAW, phase (q / RAW)
   // of this item
   auto plane_tma = [&](int p) -> bool {   // does plane p come by TMA (else loaded directly)?
@@ -970,7 +975,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
           fzd[v] = fzu[v];
         }
       }
-      if (P::GLM && glm_post) out[NV - 1] = out[NV - 1] * glm_fr;
+      if (P::GLM && glm_post) out[NV - 1] = out[NV - 1] * psi_post;
 #pragma unroll
       for (int v = 0; v < NV; ++v) Uo[base + (size_t)v * NCELL] = out[v];
       R auxk[NAW];

@@ -315,7 +315,10 @@ void HostMesh::build_descs(std::vector<BlockDesc>* desc, std::vector<GhostTask>*
         }
       }
     }
-    if (t.nface) fixups->push_back(t);
+    if (t.nface) {
+      fixups->push_back(t);
+      (*desc)[i].corrected = 1;
+    }
   }
   *nslots = ns;
 }
