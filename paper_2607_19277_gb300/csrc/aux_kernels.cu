@@ -110,6 +110,7 @@ __global__ void __launch_bounds__(256, 4) ghost_kernel(const R* __restrict__ U, 
                                                         const GhostTask* __restrict__ tasks) {
   using P = PT<R>;
   constexpr int NT = P::NV + P::NA;
+  chain_wait();
   const GhostTask& tk = tasks[blockIdx.x];
   const int d = tk.face >> 1, s = tk.face & 1;
   const int sd = axis_stride(d), st1 = d == 0 ? 16 : 1, st2 = d == 2 ? 16 : 256;
@@ -180,6 +181,7 @@ __global__ void __launch_bounds__(256) fixup_kernel(R* __restrict__ U, const R* 
                                                      const FixupTask* __restrict__ tasks, double b,
                                                      const double* __restrict__ dtch,
                                                      const int* __restrict__ solve_of) {
+  chain_wait();
   const FixupTask& tk = tasks[blockIdx.x];
   const int j = blockIdx.y, nface = tk.nface;
   if (j >= nface) return;                    // CTA-uniform
@@ -239,6 +241,7 @@ __global__ void __launch_bounds__(256) speeds_kernel(const R* __restrict__ U,
                                                       const int* __restrict__ wl) {
   using P = PT<R>;
   constexpr int NV = P::NV, NA = P::NA, NT = NV + NA;
+  chain_wait();
   const int b = wl ? wl[blockIdx.x] : (int)blockIdx.x;
   const R dxr[3] = {R(bd[b].dx[0]), R(bd[b].dx[1]), R(bd[b].dx[2])};
   R ssum = R(0), smax = R(0);
@@ -257,14 +260,17 @@ __global__ void __launch_bounds__(256) speeds_kernel(const R* __restrict__ U,
   if (st) atomicOr(status, st);
 }
 
-__global__ void set_dt_kernel(const unsigned long long* speeds, double* dtch, double dt_host,
-                              double cfl, int nsolve, double rate_floor) {
+__global__ void set_dt_kernel(unsigned long long* speeds, double* dtch, double dt_host, double cfl, int nsolve,
+                              double rate_floor, int* work, int reset) {
+  chain_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < 4) work[i] = 0;
   if (i >= nsolve) return;
   const double smax = __longlong_as_double((long long)speeds[2 * i]);
   const double cmax = __longlong_as_double((long long)speeds[2 * i + 1]);
   dtch[2 * i] = dt_host > 0.0 ? dt_host : cfl / fmax(smax, rate_floor);
   dtch[2 * i + 1] = cmax;
+  if (reset) speeds[2 * i] = speeds[2 * i + 1] = 0;
 }
 
 // ------------------------------------------------------------------------------ GLM source
@@ -276,6 +282,7 @@ __global__ void __launch_bounds__(256) glm_decay_kernel(R* __restrict__ U, const
                                                          const int* __restrict__ solve_of,
                                                          const int* __restrict__ wl) {
   __shared__ R s_f;
+  chain_wait();
   const int b = wl ? wl[blockIdx.x] : (int)blockIdx.x;
   if (threadIdx.x == 0) {
     const double* dc = dtch + 2 * (solve_of ? solve_of[b] : 0);
@@ -584,6 +591,7 @@ __global__ void __launch_bounds__(256) prim_pass_kernel(const R* __restrict__ U,
                                                         unsigned long long* speeds) {
   using P = PT<R>;
   constexpr int NV = P::NV, NA = P::NA, NT = NV + NA;
+  chain_wait();
   const int item = blockIdx.x;
   const R* src;
   R* dst;
@@ -780,6 +788,8 @@ __global__ void halo_kernel(const R* __restrict__ U, const R* __restrict__ G,
 
 cudaError_t launch_ghosts(const AuxArgs& a, const GhostTask* tasks, int ntasks, cudaStream_t s) {
   if (ntasks == 0) return cudaSuccess;
+  // not chained behind the stage kernel, nor is the fix-up: their many small CTAs, waiting where
+  // its last ones run, cost a refined blast 3-5%
 #define CALL(PT) ghost_kernel<PT, R><<<ntasks, 256, 0, s>>>((const R*)a.U, (R*)a.Gw, a.bd, tasks)
   AGILE_DISPATCH(a.phys, a.real_bytes, CALL);
 #undef CALL
@@ -792,43 +802,49 @@ cudaError_t launch_fixup(const AuxArgs& a, const FixupTask* tasks, int ntasks, d
   const int nv = phys_nvar(a.phys), nt = nv + phys_naux(a.phys);
   if (nv == 6) return cudaErrorInvalidValue;   // ffhd runs on uniform meshes only
   const dim3 grid(ntasks, NFACE);
+#define CALL(R, NV, NT) \
+  fixup_kernel<R, NV, NT><<<grid, 256, 0, s>>>((R*)a.Uw, (const R*)a.FR, a.bd, tasks, b, dtch, a.solve_of)
   if (a.real_bytes == 8) {
-    if (nv == 9) fixup_kernel<double, 9, 9><<<grid, 256, 0, s>>>((double*)a.Uw, (const double*)a.FR, a.bd, tasks, b, dtch, a.solve_of);
-    else if (nt == 5) fixup_kernel<double, 5, 5><<<grid, 256, 0, s>>>((double*)a.Uw, (const double*)a.FR, a.bd, tasks, b, dtch, a.solve_of);
-    else fixup_kernel<double, 5, 7><<<grid, 256, 0, s>>>((double*)a.Uw, (const double*)a.FR, a.bd, tasks, b, dtch, a.solve_of);
+    if (nv == 9) CALL(double, 9, 9);
+    else if (nt == 5) CALL(double, 5, 5);
+    else CALL(double, 5, 7);
   } else {
-    if (nv == 9) fixup_kernel<float, 9, 9><<<grid, 256, 0, s>>>((float*)a.Uw, (const float*)a.FR, a.bd, tasks, b, dtch, a.solve_of);
-    else if (nt == 5) fixup_kernel<float, 5, 5><<<grid, 256, 0, s>>>((float*)a.Uw, (const float*)a.FR, a.bd, tasks, b, dtch, a.solve_of);
-    else fixup_kernel<float, 5, 7><<<grid, 256, 0, s>>>((float*)a.Uw, (const float*)a.FR, a.bd, tasks, b, dtch, a.solve_of);
+    if (nv == 9) CALL(float, 9, 9);
+    else if (nt == 5) CALL(float, 5, 5);
+    else CALL(float, 5, 7);
   }
+#undef CALL
   return cudaGetLastError();
 }
 
 cudaError_t launch_speeds(const AuxArgs& a, unsigned long long* speeds, cudaStream_t s) {
   if (a.nblk == 0) return cudaSuccess;
+  cudaError_t e = cudaSuccess;
 #define CALL(PT)                                                                                  \
   do {                                                                                            \
     PhysParamsT<R> pp;                                                                            \
     pp.set(a.gamma, 0.0);                                                                         \
-    speeds_kernel<PT, R><<<dim3(a.nblk, SPEED_PARTS), 256, 0, s>>>((const R*)a.U, a.bd, pp, speeds, a.status, a.solve_of, a.wl); \
+    e = launch_chained(speeds_kernel<PT, R>, dim3(a.nblk, SPEED_PARTS), 256, 0, s, (const R*)a.U, a.bd, pp, speeds, a.status, \
+                       a.solve_of, a.wl);                                                         \
   } while (0)
   AGILE_DISPATCH(a.phys, a.real_bytes, CALL);
 #undef CALL
-  return cudaGetLastError();
+  return e;
 }
 
-cudaError_t launch_set_dt(const unsigned long long* speeds, double* dtch, double dt_host,
-                          double cfl, cudaStream_t s, int nsolve, double rate_floor) {
-  set_dt_kernel<<<(nsolve + 127) / 128, 128, 0, s>>>(speeds, dtch, dt_host, cfl, nsolve, rate_floor);
-  return cudaGetLastError();
+cudaError_t launch_set_dt(unsigned long long* speeds, double* dtch, double dt_host, double cfl, int* work,
+                          bool reset, cudaStream_t s, int nsolve, double rate_floor) {
+  return launch_chained(set_dt_kernel, dim3((nsolve + 127) / 128), 128, 0, s, speeds, dtch, dt_host, cfl, nsolve,
+                        rate_floor, work, (int)reset);
 }
 
 cudaError_t launch_glm_decay(const AuxArgs& a, const double* dtch, cudaStream_t s) {
   if (a.nblk == 0) return cudaSuccess;
   if (a.real_bytes == 8)
-    glm_decay_kernel<double><<<a.nblk, 256, 0, s>>>((double*)a.Uw, a.bd, dtch, a.glm_alpha, a.solve_of, a.wl);
-  else glm_decay_kernel<float><<<a.nblk, 256, 0, s>>>((float*)a.Uw, a.bd, dtch, a.glm_alpha, a.solve_of, a.wl);
-  return cudaGetLastError();
+    return launch_chained(glm_decay_kernel<double>, dim3(a.nblk), 256, 0, s, (double*)a.Uw, a.bd, dtch, a.glm_alpha,
+                          a.solve_of, a.wl);
+  return launch_chained(glm_decay_kernel<float>, dim3(a.nblk), 256, 0, s, (float*)a.Uw, a.bd, dtch, a.glm_alpha,
+                        a.solve_of, a.wl);
 }
 
 cudaError_t launch_estimate(const AuxArgs& a, const int* vars, const double* weights, int nvars,
@@ -856,13 +872,13 @@ cudaError_t launch_prim_pass(const AuxArgs& a, void* W, void* WG, int nslots, un
   if (grid == 0) return cudaSuccess;
   if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
   if (a.phys != PH_SRHD && a.phys != PH_SRHD_SYNGE) return cudaErrorInvalidValue;
+  cudaError_t e = cudaSuccess;
 #define CALL(PT)                                                                               \
   do {                                                                                         \
     PhysParamsT<R> pp;                                                                         \
     pp.set(a.gamma, 0.0);                                                                      \
-    prim_pass_kernel<PT, R><<<(unsigned)grid, 256, 0, s>>>((const R*)a.U, (R*)W, (const R*)a.G, \
-                                                           (R*)WG, a.wl, a.nblk, pp, a.status,   \
-                                                           a.bd, a.solve_of, speeds);            \
+    e = launch_chained(prim_pass_kernel<PT, R>, dim3((unsigned)grid), 256, 0, s, (const R*)a.U, (R*)W, \
+                       (const R*)a.G, (R*)WG, a.wl, a.nblk, pp, a.status, a.bd, a.solve_of, speeds); \
   } while (0)
   if (a.phys == PH_SRHD) {
     if (a.real_bytes == 8) { using R = double; CALL(SrhdPhys); }
@@ -872,7 +888,7 @@ cudaError_t launch_prim_pass(const AuxArgs& a, void* W, void* WG, int nslots, un
     else { using R = float; CALL(SrhdSyngePhys); }
   }
 #undef CALL
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_prim2cons(const AuxArgs& a, const double* prim, const int* blocks, int n, cudaStream_t s) {

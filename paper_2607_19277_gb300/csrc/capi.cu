@@ -712,10 +712,10 @@ agile_status agile_step(agile_mesh* m, double dt) {
   if (!lead) {
     s = ensure_speeds(m);
     if (s) return s;
-    CK(m, launch_set_dt(m->d_speeds, m->d_dtch, dt, m->cfg.cfl, m->stream, 1, mesh_res_rate(m)));
+    m->speeds_valid = false;                   // read and zeroed; the end of the step has the new ones
+    CK(m, launch_set_dt(m->d_speeds, m->d_dtch, dt, m->cfg.cfl, m->d_work, true, m->stream, 1, mesh_res_rate(m)));
     m->total_launches++;
   }
-  CK(m, cudaMemsetAsync(m->d_work, 0, 4 * sizeof(int), m->stream));
   const bool mhd = m->cfg.physics == AGILE_MHD_GLM;
   if (mhd) {
     AuxArgs a = aux_args(m, m->U[0]);
@@ -741,7 +741,6 @@ agile_status agile_step(agile_mesh* m, double dt) {
     void* Uo = last ? m->U[0] : m->U[st + 1];
     s = fill_ghosts(m, Us);
     if (s) return s;
-    if (last && speeds_in_stage) CK(m, cudaMemsetAsync(m->d_speeds, 0, 2 * sizeof(unsigned long long), m->stream));
     StageArgs A;
     A.Us = Us;
     A.Un = m->U[0];
@@ -771,7 +770,8 @@ agile_status agile_step(agile_mesh* m, double dt) {
       CK(m, launch_prim_pass(pa, m->W, m->WG, m->nslots, st == 0 ? m->d_speeds : nullptr, m->stream));
       m->total_launches++;
       if (st == 0) {
-        CK(m, launch_set_dt(m->d_speeds, m->d_dtch, dt, m->cfg.cfl, m->stream, 1, mesh_res_rate(m)));
+        CK(m, launch_set_dt(m->d_speeds, m->d_dtch, dt, m->cfg.cfl, m->d_work, false, m->stream, 1,
+                            mesh_res_rate(m)));
         m->total_launches++;
       }
       A.W = m->W;
@@ -814,7 +814,6 @@ agile_status agile_step(agile_mesh* m, double dt) {
     }
   }
   if (cool) {                                   // second half, with the CFL speeds of U^{n+1}
-    CK(m, cudaMemsetAsync(m->d_speeds, 0, 2 * sizeof(unsigned long long), m->stream));
     AuxArgs a = aux_args(m, m->U[0]);
     CK(m, launch_cooling(a, m->cool, m->d_cool, m->d_dtch, 0.5, m->d_speeds, m->stream));
     m->total_launches++;
@@ -1791,8 +1790,7 @@ agile_status batch_ensure_speeds(agile_batch* B) {
 // Enqueue one full step of every solve (device dt) on the batch stream.
 agile_status batch_enqueue_step(agile_batch* B) {
   const bool lead = B->W != nullptr;  // SRHD: dt after the first stage's recovery pass (agile_step)
-  if (!lead) BCK(B, launch_set_dt(B->d_speeds, B->d_dtch, 0.0, B->cfg.cfl, B->stream, B->nsolve));
-  BCK(B, cudaMemsetAsync(B->d_work, 0, 4 * sizeof(int), B->stream));
+  if (!lead) BCK(B, launch_set_dt(B->d_speeds, B->d_dtch, 0.0, B->cfg.cfl, B->d_work, true, B->stream, B->nsolve));
   const bool mhd = B->cfg.physics == AGILE_MHD_GLM;
   if (mhd) {
     AuxArgs a = batch_aux(B, B->U[0]);
@@ -1808,7 +1806,6 @@ agile_status batch_enqueue_step(agile_batch* B) {
       AuxArgs ga = batch_aux(B, Us);
       BCK(B, launch_ghosts(ga, B->d_ghosts, B->nghost, B->stream));
     }
-    if (last && !lead) BCK(B, cudaMemsetAsync(B->d_speeds, 0, 2 * sizeof(unsigned long long) * B->nsolve, B->stream));
     StageArgs A;
     A.Us = Us;
     A.Un = B->U[0];
@@ -1836,7 +1833,8 @@ agile_status batch_enqueue_step(agile_batch* B) {
       AuxArgs pa = batch_aux(B, Us);
       if (st == 0) BCK(B, cudaMemsetAsync(B->d_speeds, 0, 2 * sizeof(unsigned long long) * B->nsolve, B->stream));
       BCK(B, launch_prim_pass(pa, B->W, B->WG, B->nslots, st == 0 ? B->d_speeds : nullptr, B->stream));
-      if (st == 0) BCK(B, launch_set_dt(B->d_speeds, B->d_dtch, 0.0, B->cfg.cfl, B->stream, B->nsolve));
+      if (st == 0)
+        BCK(B, launch_set_dt(B->d_speeds, B->d_dtch, 0.0, B->cfg.cfl, B->d_work, false, B->stream, B->nsolve));
       A.W = B->W;
       A.WG = B->WG;
       A.tmap = &B->tmapW;
@@ -1963,7 +1961,7 @@ agile_status agile_batch_autotune(agile_batch* B, int trials, int* grid, int* dy
   if (!B || trials < 1 || trials > 100) return bfail(B, AGILE_EINVAL, "bad argument");
   agile_status s = batch_ensure_speeds(B);
   if (s) return s;
-  BCK(B, launch_set_dt(B->d_speeds, B->d_dtch, 0.0, B->cfg.cfl, B->stream, B->nsolve));
+  BCK(B, launch_set_dt(B->d_speeds, B->d_dtch, 0.0, B->cfg.cfl, B->d_work, false, B->stream, B->nsolve));
   int dev = 0, sms = 0;
   BCK(B, cudaGetDevice(&dev));
   BCK(B, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -2192,6 +2190,7 @@ agile_status agile_batch_step(agile_batch* B) {
   if (!B) return AGILE_EINVAL;
   agile_status s = B->W ? AGILE_OK : batch_ensure_speeds(B);   // SRHD: the first pass reduces them
   if (s) return s;
+  B->speeds_valid = false;    // the step reads and zeroes them; its end has the new ones
   if (B->steps_done == 0) {   // first step eagerly: sets kernel attributes outside any capture
     s = batch_enqueue_step(B);
     if (s) return s;

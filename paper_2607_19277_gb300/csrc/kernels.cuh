@@ -106,6 +106,14 @@ __device__ __forceinline__ void load_cell(const R* __restrict__ U, const R* __re
   for (int v = 0; v < NT; ++v) u[v] = p[(size_t)v * NCELL];
 }
 
+// Chained launches (launch_chained): wait until the kernel before this one on the stream has
+// completed and its writes are visible (nothing to wait for in a plain launch), then let the
+// next one take its place.
+__device__ __forceinline__ void chain_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 __device__ __forceinline__ void atomic_max_pos(unsigned long long* addr, double v) {
   atomicMax(addr, (unsigned long long)__double_as_longlong(v));
 }
@@ -414,6 +422,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
     for (int i = 0; i < RAW; ++i) mbar_init(bar + i, 1);
     fence_mbar_init();
   }
+  chain_wait();
   __syncthreads();
   int st = 0;
   // Persistent loop: this CTA starts with item blockIdx.x and then takes the next free item

@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <utility>
 #include <vector>
 
 #include "agile_internal.h"
@@ -9,6 +10,29 @@
 namespace agile {
 
 struct StageArgs;
+
+// Launch of a step's kernel behind the kernel before it on the stream, allowed to start while
+// that one drains (programmatic stream serialisation): its CTAs take their places and set up
+// shared memory, then wait (chain_wait in the kernel, before its first access of global memory)
+// until the kernel before has completed. Behind anything but a kernel it is a plain launch. Saves
+// the gap between dependent launches: with the two memsets of a step gone as well (set_dt), a
+// step of 30 MHD blocks in FP32 takes 45 us instead of 56, a host-timed step of 8 FP64 HD blocks
+// 167 instead of 179.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_chained(void (*k)(KArgs...), dim3 grid, unsigned block, size_t smem, cudaStream_t s,
+                           Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...);
+}
 
 // Per-stage update (macro-kernel), dispatched on physics / precision / limiter / flux.
 cudaError_t launch_stage_hd(int real_bytes, int lim, int flux, const StageArgs& a, cudaStream_t s);
@@ -56,9 +80,10 @@ cudaError_t launch_fixup(const AuxArgs& a, const FixupTask* tasks, int ntasks, d
 // Max signal-speed reduction of U into speeds[2] (double bits; caller zeroes them).
 cudaError_t launch_speeds(const AuxArgs& a, unsigned long long* speeds, cudaStream_t s);
 // dtch[solve] = {dt, c_h}: dt from the host value or (dt <= 0) cfl / max sum_d s_d / dx_d,
-// for each of nsolve solves (speeds[solve][2]).
-cudaError_t launch_set_dt(const unsigned long long* speeds, double* dtch, double dt_host,
-                          double cfl, cudaStream_t s, int nsolve = 1, double rate_floor = 0.0);
+// for each of nsolve solves (speeds[solve][2]). Also zeroes the step's block counters work[4]
+// and, with reset, the speeds it has read, for the reduction at the end of the step.
+cudaError_t launch_set_dt(unsigned long long* speeds, double* dtch, double dt_host, double cfl, int* work,
+                          bool reset, cudaStream_t s, int nsolve = 1, double rate_floor = 0.0);
 // psi *= exp(-dt/2 c_h alpha / min dx) on every block.
 cudaError_t launch_glm_decay(const AuxArgs& a, const double* dtch, cudaStream_t s);
 // Loehner estimate: emax[nblk] (FP64, no FMA). With tols (per solve {refine threshold,

@@ -1,6 +1,7 @@
 // Launch of the persistent per-stage update kernel for one physics trait and scheme.
 #pragma once
 #include "kernels.cuh"
+#include "launch.h"
 
 namespace agile {
 
@@ -76,9 +77,7 @@ static cudaError_t stage_go_layout(const StageArgs& a, cudaStream_t s) {
   args.fb = (float)a.b;
   args.combine = a.a != 0.0 ? 1 : 0;
   const CUtensorMap& tm = *static_cast<const CUtensorMap*>(args.tmap);
-  if (args.zs) cut<<<grid, 256, SMEM, s>>>(tm, args);
-  else whole<<<grid, 256, SMEM, s>>>(tm, args);
-  return cudaGetLastError();
+  return launch_chained(args.zs ? cut : whole, dim3(grid), 256, SMEM, s, tm, args);
 }
 
 // Staging layouts: STAGE_LAYOUT_RING4 = four raw slots, one flux buffer, two barriers per
