@@ -776,6 +776,14 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
     }
     // U^n of cell (tx, ty, k) for the stage combine, loaded now so that the face work of
     // this phase covers its latency
+    // likewise U_s of the cell where the ring holds primitives from the recovery pass (read at
+    // the update it held up every plane: 332 -> 317 us a launch of 1584 FP32 blocks)
+    R usk[PRIMIN ? NV : 1];
+    if constexpr (PRIMIN) {
+      const R* ps = Us + (size_t)b * NT * NCELL + (size_t)k * 256 + cell2;
+#pragma unroll
+      for (int v = 0; v < NV; ++v) usk[v] = __ldg(ps + (size_t)v * NCELL);
+    }
     R unk[NV];
     if (combine) {
       const R* pn = Un + (size_t)b * NT * NCELL + (size_t)k * 256 + cell2;
@@ -978,7 +986,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
             if (v >= P::BOFF && v < P::BOFF + 3) L = L + rsrc[v - P::BOFF];
             if (v == P::IE) L = L + rsrc[3];
           }
-          R val = raw[(size_t)v * RSTR] + rdt * L;
+          R val = (PRIMIN ? usk[PRIMIN ? v : 0] : raw[(size_t)v * RSTR]) + rdt * L;
           if (combine) val = ra * unk[v] + rb * val;
           out[v] = val;
           fzd[v] = fzu[v];
