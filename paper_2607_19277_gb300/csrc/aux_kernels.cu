@@ -636,16 +636,21 @@ __global__ void __launch_bounds__(256) prim_pass_kernel(const R* __restrict__ U,
 }
 
 // ------------------------------------------------------------------------------ state I/O
+// Four CTAs (grid.y) per block. The conversion runs in FP64 whatever the stencil precision, and
+// the FP64 units bind it: the equation parameters come from the host, Gamma is formed once and
+// xi = Gamma^2 rho h from the conserved values it has just been part of, xi = tau + p + D.
+constexpr int IC_PARTS = 4;
 template <template <typename> class PT, typename R>
-__global__ void prim2cons_kernel(R* __restrict__ U, const double* __restrict__ prim,
-                                 const int* __restrict__ blocks, double gamma) {
+__global__ void __launch_bounds__(256) prim2cons_kernel(R* __restrict__ U, const double* __restrict__ prim,
+                                                         const int* __restrict__ blocks,
+                                                         const PhysParamsT<double> pp) {
   using P = PT<double>;
   constexpr int NV = P::NV, NA = P::NA, NT = NV + NA;
   const int i = blockIdx.x;
   const int b = blocks[i];
-  PhysParamsT<double> pp;
-  pp.set(gamma, 0.0);
-  for (int c = threadIdx.x; c < NCELL; c += blockDim.x) {
+#pragma unroll 2
+  for (int j = 0; j < NCELL / IC_PARTS / 256; ++j) {
+    const int c = blockIdx.y * (NCELL / IC_PARTS) + j * 256 + threadIdx.x;
     double p[NV], u[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) p[v] = prim[((size_t)i * NV + v) * NCELL + c];
@@ -654,11 +659,8 @@ __global__ void prim2cons_kernel(R* __restrict__ U, const double* __restrict__ p
 #pragma unroll
     for (int v = 0; v < NV; ++v) o[(size_t)v * NCELL] = R(u[v]);
     if constexpr (NA > 0) {
-      // xi = Gamma^2 rho h and Gamma from the primitives (Eq. 20)
-      const double lor = sqrt(1.0 + p[1] * p[1] + p[2] * p[2] + p[3] * p[3]);
-      const double h = P::enthalpy(p[0], p[4], pp);
-      o[(size_t)NV * NCELL] = R(lor * lor * p[0] * h);
-      o[(size_t)(NV + 1) * NCELL] = R(lor);
+      o[(size_t)NV * NCELL] = R((u[4] + p[4]) + u[0]);
+      o[(size_t)(NV + 1) * NCELL] = R(rsqrt_(1.0 + p[1] * p[1] + p[2] * p[2] + p[3] * p[3]));
     }
   }
 }
@@ -893,7 +895,9 @@ cudaError_t launch_prim_pass(const AuxArgs& a, void* W, void* WG, int nslots, un
 
 cudaError_t launch_prim2cons(const AuxArgs& a, const double* prim, const int* blocks, int n, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
-#define CALL(PT) prim2cons_kernel<PT, R><<<n, 256, 0, s>>>((R*)a.Uw, prim, blocks, a.gamma)
+  PhysParamsT<double> pp;
+  pp.set(a.gamma, 0.0);
+#define CALL(PT) prim2cons_kernel<PT, R><<<dim3(n, IC_PARTS), 256, 0, s>>>((R*)a.Uw, prim, blocks, pp)
   AGILE_DISPATCH(a.phys, a.real_bytes, CALL);
 #undef CALL
   return cudaGetLastError();
