@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   constexpr bool US_GLOBAL = RAW == 3 || PRIMIN;   // the update reads U_s of its cell from global memory
   using S = StageSmem<PT, R, RAW, SFB>;
   constexpr int NV = P::NV, NA = P::NA, NT = NV + NA;
-  // FP32 HD / MHD with HLL or TVDLF: x- and y-faces solved as packed pairs
+  // FP32 with HLL or TVDLF: x- and y-faces solved as packed pairs
   constexpr bool PAIRED = sizeof(R) == 4 && PairPhys<P>::OK && (FLUX == FLUX_HLL || FLUX == FLUX_TVDLF);
   constexpr int NAW = NA > 0 ? NA : 1;
   constexpr bool RESP = res_of<P>::value;   // resistive MHD sources

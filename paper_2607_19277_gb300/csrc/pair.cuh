@@ -6,8 +6,8 @@
 // instructions of the sm_100 family (add / sub / mul / fma .f32x2: one issue, two results).
 // Reciprocals, square roots, minima, maxima and selects act on each half. The pair forms
 // below restate, for the x direction, the face states (PLM, Section 2.1.1), the primitive-to-
-// conserved map, physical fluxes and signal speeds of HD (Section 2.3.1, Eqs. 2-6) and MHD
-// with GLM (Section 2.3.3, Eqs. 11-14) and the HLL / TVDLF fluxes of the scalar solver; their
+// conserved map, physical fluxes and signal speeds of HD (Section 2.3.1, Eqs. 2-6), MHD with GLM
+// (Section 2.3.3, Eqs. 11-14), FFHD and SRHD and the HLL / TVDLF fluxes of the scalar solver; their
 // products and sums are contracted into fused multiply-adds in places where the scalar code
 // rounds separately, so a face flux agrees with the scalar solver's to a few FP32 ulps.
 #pragma once
@@ -120,9 +120,10 @@ __device__ __forceinline__ void plm2(const f2* a, const f2* b, const f2* c, cons
 
 // Constants of the pair solvers, broadcast to both halves.
 struct PairK {
-  f2 zero, half, gamma, g1, ig1, m4, ch2, nhich, nhch;
+  f2 zero, half, one, gamma, g1, ig1, gg1, m4, ch2, nhich, nhch;
   __device__ __forceinline__ explicit PairK(const PhysParamsT<float>& pp)
-      : zero(bc2(0.0f)), half(bc2(0.5f)), gamma(bc2(pp.gamma)), g1(bc2(pp.g1)), ig1(bc2(pp.ig1)),
+      : zero(bc2(0.0f)), half(bc2(0.5f)), one(bc2(1.0f)), gamma(bc2(pp.gamma)), g1(bc2(pp.g1)),
+        ig1(bc2(pp.ig1)), gg1(bc2(pp.gg1)),
         m4(bc2(-4.0f)), ch2(bc2(pp.ch2)), nhich(bc2(-0.5f * pp.ich)), nhch(bc2(-0.5f * pp.ch)) {}
 };
 
@@ -263,6 +264,64 @@ struct PairPhys<FfhdPhysT<float, HTC>> {
     const f2 w = c * abs2(p[B]);
     lm = a - w;
     lp = a + w;
+  }
+};
+
+// Special-relativistic hydrodynamics (Section 2.3.4, Eqs. 15-22) in the x direction, the formulas
+// of the scalar trait's side(): one root and one quotient for Gamma, shared by the three functions
+// (the compiler merges the repeated expressions). Recovery pass and stage over 1584 blocks: 319 us
+// with the scalar solver, 309 with pairs.
+template <int EOS>
+struct PairPhys<SrhdPhysE<float, EOS>> {
+  static constexpr bool OK = true;
+  static constexpr int NV = 5;
+  __host__ __device__ static constexpr int zrot(int v) { return v == 1 ? 3 : v == 3 ? 1 : v; }
+  __device__ static __forceinline__ void interface(f2*, f2*, const PairK&) {}
+  __device__ static __forceinline__ f2 gam(const f2* p, const PairK& k) {
+    return sqrt2(fma2(p[3], p[3], fma2(p[2], p[2], fma2(p[1], p[1], k.one))));
+  }
+  // rho h and the squared sound speed
+  __device__ static __forceinline__ void closure(const f2* p, f2& w, f2& cs2, const PairK& k) {
+    if constexpr (EOS == EOS_SYNGE) {
+      const f2 th = p[4] * rcp2(p[0]);
+      const f2 h = fma2(bc2(2.5f), th, sqrt2(fma2(bc2(2.25f) * th, th, k.one)));
+      w = p[0] * h;
+      cs2 = th * (bc2(5.0f) * h - bc2(8.0f) * th) * rcp2(bc2(3.0f) * h * (h - th));
+    } else {
+      w = fma2(k.gg1, p[4], p[0]);
+      cs2 = k.gamma * p[4] * rcp2(w);
+    }
+  }
+  __device__ static __forceinline__ void prim2cons(const f2* p, f2* u, const PairK& k) {
+    const f2 lor = gam(p, k);
+    f2 w, cs2;
+    closure(p, w, cs2, k);
+    const f2 lr = lor * p[0], lw = lor * w;
+    u[0] = lr;
+    u[1] = lw * p[1];
+    u[2] = lw * p[2];
+    u[3] = lw * p[3];
+    u[4] = (lor * lw - p[4]) - lr;
+  }
+  __device__ static __forceinline__ void flux(const f2* p, const f2* u, f2* f, const PairK& k) {
+    const f2 vd = p[1] * rcp2(gam(p, k));
+    f[0] = u[0] * vd;
+    f[1] = fma2(u[1], vd, p[4]);
+    f[2] = u[2] * vd;
+    f[3] = u[3] * vd;
+    f[4] = u[1] - f[0];
+  }
+  __device__ static __forceinline__ void lambdas(const f2* p, f2& lm, f2& lp, const PairK& k) {
+    const f2 il = rcp2(gam(p, k));
+    const f2 vd = p[1] * il;
+    f2 w, cs2;
+    closure(p, w, cs2, k);
+    const f2 il2 = il * il;                       // 1 - v^2
+    const f2 den = k.one - (k.one - il2) * cs2, a = vd * (k.one - cs2);
+    const f2 root = sqrt2(max2(cs2 * il2 * (den - vd * a), k.zero));
+    const f2 iden = rcp2(den);
+    lm = (a - root) * iden;
+    lp = (a + root) * iden;
   }
 };
 
