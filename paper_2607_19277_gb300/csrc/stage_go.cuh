@@ -19,22 +19,24 @@ constexpr int stage_minb() {
 // Work items per block: a launch of few blocks is cut along z into 2^zs items of 16 >> zs planes
 // each, so that it fills the SMs (one block per CTA leaves 144 of 152 SMs idle at 8 blocks and
 // runs 16 planes in sequence). An item costs its planes and a start c (four more planes
-// loaded and converted, one more z-face) of about c = 1.1 planes in FP32 and 0.5 in FP64, whose
-// faces cost more; the SM with the most items decides, and an item alone on its SM runs slower
-// per plane than several together (by 1.4 in FP32, by 1.09 in FP64 where two CTAs fit). The
-// smallest cost by this count, whole blocks unless a cut is at least 3% better, is within 5%
-// of the fastest cut in all 13 sizes x 7 schemes timed. us per stage launch on 152 SMs, whole
-// blocks -> chosen cut: HD FP64 8 blocks 714 -> 69, 64 blocks 718 -> 356, 512 blocks 2560 ->
-// 2341; MHD FP32 8 blocks 49 -> 14, 64 blocks 50 -> 29, 210 blocks 78 -> 64, 1000 blocks 243
-// uncut (256 cut in two).
-inline int stage_zsplit(int nblk, int sms, bool fp64, int ctas_per_sm) {
-  const double c = fp64 ? 0.5 : 1.1;
-  const double lone = fp64 ? (ctas_per_sm > 1 ? 1.09 : 1.0) : 1.4;
+// loaded and converted, one more z-face) of about c = 1.1 planes in FP32, 0.6 where the planes
+// come as primitives (SRHD) and 0.5 in FP64, whose faces cost more; the SM with the most items
+// decides, and few items on an SM run slower per plane than a full one: one alone by 1.4 in FP32
+// and by 1.12 in FP64 where two CTAs fit, two of three by 1.15 for SRHD in FP32. The smallest
+// cost by this count, whole blocks unless a cut is at least 3% better, is within 4% of the
+// fastest cut in 16 sizes x 7 schemes timed (SRHD in FP32 within 13%). us per stage launch on
+// 152 SMs, whole blocks -> chosen cut: HD FP64 8 blocks 633 -> 64, 64 blocks 635 -> 323, 512
+// blocks 2301 -> 2098; MHD FP32 8 blocks 47 -> 13, 64 blocks 48 -> 27, 210 blocks 73 -> 61, 1000
+// blocks 230 uncut (242 cut in two).
+inline int stage_zsplit(int nblk, int sms, bool fp64, bool prims, int ctas_per_sm) {
+  const double c = fp64 ? 0.5 : (prims ? 0.6 : 1.1);
+  const double one = fp64 ? (ctas_per_sm > 1 ? 1.12 : 1.0) : 1.4;
+  const double two = !fp64 && prims ? 1.15 : 1.0;
   int best = 0;
   double best_cost = 0.0;
   for (int zs = 0; zs <= 4; ++zs) {
     const long long per_sm = (((long long)nblk << zs) + sms - 1) / sms;
-    const double cost = (double)per_sm * ((NB >> zs) + c) * (per_sm == 1 ? lone : 1.0);
+    const double cost = (double)per_sm * ((NB >> zs) + c) * (per_sm == 1 ? one : per_sm == 2 ? two : 1.0);
     if (zs == 0 || cost < 0.97 * best_cost) {
       best = zs;
       best_cost = cost;
@@ -69,7 +71,7 @@ static cudaError_t stage_go_layout(const StageArgs& a, cudaStream_t s) {
   }
   if (a.nblk <= 0) return cudaSuccess;
   StageArgs args = a;
-  args.zs = Z_CUT ? stage_zsplit(a.nblk, sms, sizeof(R) == 8, MINB) : 0;
+  args.zs = Z_CUT ? stage_zsplit(a.nblk, sms, sizeof(R) == 8, prim_pass_of<PT<R>>::value, MINB) : 0;
   int grid = a.grid > 0 ? a.grid : MINB * sms;   // a tuned persistent grid, else the default
   if (grid > (a.nblk << args.zs)) grid = a.nblk << args.zs;
   args.ppf.set(a.gamma, 0.0);
