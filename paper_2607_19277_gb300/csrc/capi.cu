@@ -260,11 +260,17 @@ agile_status make_tmap(agile_mesh* m, void* U, CUtensorMap* out) {
 
 // (Re)build descriptors, slots and scratch for the current host mesh; U[0] must already
 // hold nblk blocks.
-// 2-D Morton code of (x, y) (16 bits each).
+// 2-D Morton code of (x, y) (16 bits each): the bit strings spread by halves.
 uint64_t morton2(uint32_t x, uint32_t y) {
-  uint64_t c = 0;
-  for (int i = 0; i < 16; ++i) c |= (uint64_t)((x >> i) & 1) << (2 * i) | (uint64_t)((y >> i) & 1) << (2 * i + 1);
-  return c;
+  auto spread = [](uint32_t v) {
+    uint64_t q = v & 0xffffu;
+    q = (q | (q << 8)) & 0x00ff00ffull;
+    q = (q | (q << 4)) & 0x0f0f0f0full;
+    q = (q | (q << 2)) & 0x33333333ull;
+    q = (q | (q << 1)) & 0x55555555ull;
+    return q;
+  };
+  return spread(x) | spread(y) << 1;
 }
 
 // Order in which the stage kernel's persistent CTAs take the blocks: by level, then by z
@@ -273,16 +279,20 @@ uint64_t morton2(uint32_t x, uint32_t y) {
 // slabs just before and after it, which keeps the halo re-reads in L2 (the pool itself stays
 // in 3-D Morton order).
 std::vector<int> slab_order(const HostMesh& hm) {
+  struct Slab {
+    uint64_t slab, code;             // level and z, 2-D Morton code: formed once per block
+    int at;
+    bool operator<(const Slab& o) const { return slab != o.slab ? slab < o.slab : code < o.code; }
+  };
   const auto& keys = hm.blocks();
+  std::vector<Slab> order(keys.size());
+  for (size_t i = 0; i < keys.size(); ++i) {
+    const Key& k = keys[i];
+    order[i] = {(uint64_t)k.lev << 32 | (uint32_t)k.z, morton2((uint32_t)k.x, (uint32_t)k.y), (int)i};
+  }
+  std::stable_sort(order.begin(), order.end());
   std::vector<int> w(keys.size());
-  for (size_t i = 0; i < keys.size(); ++i) w[i] = (int)i;
-  std::stable_sort(w.begin(), w.end(), [&](int a, int b) {
-    const Key& p = keys[a];
-    const Key& q = keys[b];
-    if (p.lev != q.lev) return p.lev < q.lev;
-    if (p.z != q.z) return p.z < q.z;
-    return morton2(p.x, p.y) < morton2(q.x, q.y);
-  });
+  for (size_t i = 0; i < keys.size(); ++i) w[i] = order[i].at;
   return w;
 }
 

@@ -4,23 +4,36 @@
 #include "mesh.h"
 
 #include <algorithm>
+#include <array>
 #include <deque>
 
 namespace agile {
 
-uint64_t morton3(uint32_t x, uint32_t y, uint32_t z) {
-  uint64_t m = 0;
-  for (int b = 0; b < 21; ++b) {
-    m |= (uint64_t)((x >> b) & 1u) << (3 * b);
-    m |= (uint64_t)((y >> b) & 1u) << (3 * b + 1);
-    m |= (uint64_t)((z >> b) & 1u) << (3 * b + 2);
-  }
-  return m;
+// The low 21 bits of v, two zero bits after each: halves of the bit string move apart by twice
+// their length, step by step.
+static uint64_t spread3(uint32_t v) {
+  uint64_t x = v & 0x1fffffu;
+  x = (x | (x << 32)) & 0x001f00000000ffffull;
+  x = (x | (x << 16)) & 0x001f0000ff0000ffull;
+  x = (x | (x << 8)) & 0x100f00f00f00f00full;
+  x = (x | (x << 4)) & 0x10c30c30c30c30c3ull;
+  x = (x | (x << 2)) & 0x1249249249249249ull;
+  return x;
 }
 
-static bool key_less(const Key& a, const Key& b) {
-  if (a.lev != b.lev) return a.lev < b.lev;
-  return morton3(a.x, a.y, a.z) < morton3(b.x, b.y, b.z);
+uint64_t morton3(uint32_t x, uint32_t y, uint32_t z) {
+  return spread3(x) | spread3(y) << 1 | spread3(z) << 2;
+}
+
+// Order of the blocks, formed once per block: level, then Morton index; with the block's place.
+struct OrderKey {
+  uint64_t code;
+  int lev;
+  int at;
+  bool operator<(const OrderKey& o) const { return lev != o.lev ? lev < o.lev : code < o.code; }
+};
+static OrderKey order_key(const Key& k, int at) {
+  return {morton3((uint32_t)k.x, (uint32_t)k.y, (uint32_t)k.z), k.lev, at};
 }
 
 HostMesh::HostMesh(const int base[3], int max_level, const int bc[6], const double xmin[3],
@@ -36,20 +49,23 @@ HostMesh::HostMesh(const int base[3], int max_level, const int bc[6], const doub
   for (int z = 0; z < base[2]; ++z)
     for (int y = 0; y < base[1]; ++y)
       for (int x = 0; x < base[0]; ++x) blocks_.push_back(Key{1, x, y, z});
+  std::vector<OrderKey> order;
+  order.reserve(blocks_.size());
+  for (size_t i = 0; i < blocks_.size(); ++i) order.push_back(order_key(blocks_[i], (int)i));
+  std::sort(order.begin(), order.end());
+  std::vector<Key> sorted;
+  sorted.reserve(blocks_.size());
+  for (const OrderKey& o : order) sorted.push_back(blocks_[o.at]);
+  blocks_.swap(sorted);
   reindex();
 }
 
-void HostMesh::reindex() {
-  std::sort(blocks_.begin(), blocks_.end(), key_less);
-  index_.clear();
-  index_.reserve(blocks_.size() * 2);
-  for (size_t i = 0; i < blocks_.size(); ++i) index_[key_code(blocks_[i])] = (int)i;
+void HostMesh::reindex() {           // blocks_ is in order
+  index_.reset(blocks_.size());
+  for (size_t i = 0; i < blocks_.size(); ++i) index_.insert(key_code(blocks_[i]), (int)i);
 }
 
-int HostMesh::find(const Key& k) const {
-  auto it = index_.find(key_code(k));
-  return it == index_.end() ? -1 : it->second;
-}
+int HostMesh::find(const Key& k) const { return index_.find(key_code(k)); }
 
 double HostMesh::dx(int lev, int d) const {
   return (xmax_[d] - xmin_[d]) / ((double)base_[d] * NB * (double)(1 << (lev - 1)));
@@ -152,12 +168,12 @@ RegridPlan HostMesh::plan(const std::vector<int>& flags) const {
         }
   }
   // Nodes with children after refinement.
-  std::unordered_set<uint64_t> internal;
+  KeyTable internal(n);
   for (int i = 0; i < n; ++i) {
     Key q = blocks_[i];
     while (q.lev > 1) {
       q = Key{q.lev - 1, q.x >> 1, q.y >> 1, q.z >> 1};
-      if (!internal.insert(key_code(q)).second) break;
+      if (!internal.insert(key_code(q))) break;
     }
     if (refine[i]) internal.insert(key_code(blocks_[i]));
   }
@@ -165,14 +181,15 @@ RegridPlan HostMesh::plan(const std::vector<int>& flags) const {
   // and no block adjacent to the parent refined in the post-refinement tree.
   std::vector<char> coarsen(n, 0);
   std::vector<Key> new_parents;
-  std::vector<std::vector<int>> parent_kids;
-  std::unordered_set<uint64_t> seen;
+  std::vector<std::array<int, 8>> parent_kids;
+  KeyTable seen(n);
   for (int i = 0; i < n; ++i) {
     const Key& k = blocks_[i];
     if (k.lev < 2) continue;
     const Key pk{k.lev - 1, k.x >> 1, k.y >> 1, k.z >> 1};
-    if (!seen.insert(key_code(pk)).second) continue;
-    std::vector<int> kids(8, -1);
+    if (!seen.insert(key_code(pk))) continue;
+    std::array<int, 8> kids;
+    kids.fill(-1);
     bool ok = true;
     for (int o = 0; o < 8 && ok; ++o) {
       const int j = find(Key{k.lev, 2 * pk.x + (o & 1), 2 * pk.y + ((o >> 1) & 1),
@@ -190,7 +207,7 @@ RegridPlan HostMesh::plan(const std::vector<int>& flags) const {
             Key q;
             if (!neighbour_pos(c, ox, oy, oz, &q)) continue;
             if ((q.x >> 1) == pk.x && (q.y >> 1) == pk.y && (q.z >> 1) == pk.z) continue;
-            if (internal.count(key_code(q))) ok = false;
+            if (internal.find(key_code(q)) >= 0) ok = false;
           }
     }
     if (!ok) continue;
@@ -205,6 +222,7 @@ RegridPlan HostMesh::plan(const std::vector<int>& flags) const {
     bool created;
   };
   std::vector<Item> items;
+  items.reserve(n + 7 * (size_t)std::count(refine.begin(), refine.end(), 1));
   for (int i = 0; i < n; ++i) {
     const Key& k = blocks_[i];
     if (refine[i]) {
@@ -238,11 +256,17 @@ RegridPlan HostMesh::plan(const std::vector<int>& flags) const {
     items.push_back(it);
   }
   P.n_coarsened = (int)new_parents.size();
-  std::sort(items.begin(), items.end(), [](const Item& a, const Item& b) { return key_less(a.k, b.k); });
+  std::vector<OrderKey> order;
+  order.reserve(items.size());
+  for (size_t i = 0; i < items.size(); ++i) order.push_back(order_key(items[i].k, (int)i));
+  std::sort(order.begin(), order.end());
+  P.blocks.reserve(items.size());
+  P.src.reserve(items.size());
   for (size_t i = 0; i < items.size(); ++i) {
-    P.blocks.push_back(items[i].k);
-    P.src.push_back(items[i].s);
-    if (items[i].created) P.created.push_back((int)i);
+    const Item& it = items[order[i].at];
+    P.blocks.push_back(it.k);
+    P.src.push_back(it.s);
+    if (it.created) P.created.push_back((int)i);
   }
   return P;
 }
@@ -259,7 +283,7 @@ void HostMesh::build_descs(std::vector<BlockDesc>* desc, std::vector<GhostTask>*
   ghosts->clear();
   fixups->clear();
   int ns = 0;
-  std::vector<FaceInfo> fis((size_t)n * 6);
+  ghosts->reserve(n);
   for (int i = 0; i < n; ++i) {
     BlockDesc& bd = (*desc)[i];
     const Key& k = blocks_[i];
@@ -267,7 +291,6 @@ void HostMesh::build_descs(std::vector<BlockDesc>* desc, std::vector<GhostTask>*
     for (int d = 0; d < 3; ++d) bd.dx[d] = dx(k.lev, d);
     for (int f = 0; f < 6; ++f) {
       const FaceInfo fi = face(i, f);
-      fis[(size_t)i * 6 + f] = fi;
       bd.kind[f] = fi.kind;
       bd.slot[f] = -1;
       for (int q = 0; q < 4; ++q) bd.nbr[f][q] = fi.nbr[q];

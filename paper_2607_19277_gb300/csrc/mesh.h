@@ -5,8 +5,6 @@
 #include <stdint.h>
 
 #include <string>
-#include <unordered_map>
-#include <unordered_set>
 #include <vector>
 
 #include "agile_internal.h"
@@ -23,6 +21,58 @@ inline uint64_t key_code(const Key& k) {
 }
 
 uint64_t morton3(uint32_t x, uint32_t y, uint32_t z);
+
+// Open-addressing table from key codes (never 0: levels start at 1) to integers, in two flat
+// arrays at most half full: a regrid builds and asks such tables tens of thousands of times.
+class KeyTable {
+ public:
+  explicit KeyTable(size_t n = 0) { reset(n); }
+  void reset(size_t n) {             // empty, with room for n keys
+    size_t cap = 64;
+    shift_ = 64 - 6;
+    while (cap < 2 * n) {
+      cap *= 2;
+      --shift_;
+    }
+    keys_.assign(cap, 0);
+    vals_.assign(cap, 0);
+    size_ = 0;
+  }
+  bool insert(uint64_t code, int val = 0) {   // false when the key is there already
+    if (2 * (size_ + 1) > keys_.size()) grow();
+    const size_t i = slot(code);
+    if (keys_[i]) return false;
+    keys_[i] = code;
+    vals_[i] = val;
+    ++size_;
+    return true;
+  }
+  int find(uint64_t code) const {    // its value, -1 without the key
+    const size_t i = slot(code);
+    return keys_[i] ? vals_[i] : -1;
+  }
+
+ private:
+  size_t slot(uint64_t code) const {  // where the key is or would be
+    const size_t mask = keys_.size() - 1;
+    size_t i = (size_t)((code * 0x9E3779B97F4A7C15ull) >> shift_);   // the product's high bits
+    while (keys_[i] && keys_[i] != code) i = (i + 1) & mask;
+    return i;
+  }
+  void grow() {
+    std::vector<uint64_t> k;
+    std::vector<int> v;
+    k.swap(keys_);
+    v.swap(vals_);
+    reset(k.size());
+    for (size_t i = 0; i < k.size(); ++i)
+      if (k[i]) insert(k[i], v[i]);
+  }
+  std::vector<uint64_t> keys_;
+  std::vector<int> vals_;
+  size_t size_ = 0;
+  int shift_ = 0;
+};
 
 struct FaceInfo {
   int kind;      // FK_*
@@ -73,7 +123,7 @@ class HostMesh {
   bool periodic_[3];
   double xmin_[3], xmax_[3];
   std::vector<Key> blocks_;
-  std::unordered_map<uint64_t, int> index_;
+  KeyTable index_;
 };
 
 }  // namespace agile
