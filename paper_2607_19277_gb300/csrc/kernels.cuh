@@ -313,14 +313,19 @@ __device__ __forceinline__ int pslot(int p) { return (p + 3) % 3; }
 template <template <typename> class PT, typename R, int RAW, int SFB>
 struct StageSmem {
   static constexpr int NV = PT<R>::NV, NT = PT<R>::NV + PT<R>::NA;
-  // x-face fluxes: row r, faces 0 .. 16; y-face fluxes: faces 0 .. 16, column c. FP32 rows are 20
-  // wide, so that a warp's two rows (r, r + 4) lie 16 banks apart; FP64 rows (a half-warp covers
-  // the banks) 16, the last x-face of each row after the others.
-  static constexpr int FP = sizeof(R) == 4 ? 20 : 16;
+  // x-face fluxes: row r, faces 0 .. 16; y-face fluxes: face 0 .. 16, 16 columns. In FP32 a warp's
+  // two rows (r, r + 4) are to lie 16 banks apart: rows 20 wide, or with three raw slots (where
+  // that space decides whether two CTAs fit: MHD) y rows 16 wide of which those with bit 2 set
+  // change places in pairs. In FP64 (a half-warp covers the banks) plain rows of 16, the last
+  // x-face of each row after the others.
+  static constexpr bool SWAP = sizeof(R) == 4 && RAW == 3;
   static constexpr int FXN = sizeof(R) == 4 ? 16 * 20 : 272;
-  static constexpr int FYN = sizeof(R) == 4 ? 16 * 20 + 16 : 272;
+  static constexpr int FYN = sizeof(R) == 4 && !SWAP ? 16 * 20 + 16 : 272;
   __host__ __device__ static constexpr int xf(int r, int f) {
-    return sizeof(R) == 4 || f < 16 ? r * FP + f : 256 + r;
+    return sizeof(R) == 4 ? r * 20 + f : (f < 16 ? r * 16 + f : 256 + r);
+  }
+  __host__ __device__ static constexpr int yf(int f, int c) {
+    return SWAP ? (f ^ ((f >> 2) & 1)) * 16 + c : f * (sizeof(R) == 4 ? 20 : 16) + c;
   }
   static constexpr size_t bars = 128;                                  // RAW mbarriers (+pad)
   static constexpr size_t raw = bars;                                  // [RAW][NT][256]
@@ -404,9 +409,9 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   const int cell2 = ty * 16 + tx;
   const int cellp = (ty + 2) * 20 + tx + 2;   // this thread's cell in a 20 x 20 ring plane
   // slots of its lower and upper x- and y-face in the flux buffers
-  constexpr int FP = S::FP, FXN = S::FXN, FYN = S::FYN;
+  constexpr int FXN = S::FXN, FYN = S::FYN;
   const int fx0 = S::xf(ty, tx), fx1 = S::xf(ty, tx + 1);
-  const int fy0 = ty * FP + tx, fy1 = fy0 + FP;
+  const int fy0 = S::yf(ty, tx), fy1 = S::yf(ty + 1, tx);
   // Halo cell of this thread: h < 64 x-faces, above y-faces; the half t >> 7 of the CTA owns
   // the halo of the planes of its parity.
   const int hh = t & 127;
@@ -776,10 +781,10 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
     }
     // U^n of cell (tx, ty, k) for the stage combine, loaded now so that the face work of
     // this phase covers its latency
-    // likewise U_s of the cell where the ring holds primitives from the recovery pass (read at
-    // the update it held up every plane: 332 -> 317 us a launch of 1584 FP32 blocks)
-    R usk[PRIMIN ? NV : 1];
-    if constexpr (PRIMIN) {
+    // likewise U_s of the cell where no raw plane holds it then (read at the update it held up
+    // every plane: SRHD 332 -> 317 us a launch of 1584 FP32 blocks)
+    R usk[US_GLOBAL ? NV : 1];
+    if constexpr (US_GLOBAL) {
       const R* ps = Us + (size_t)b * NT * NCELL + (size_t)k * 256 + cell2;
 #pragma unroll
       for (int v = 0; v < NV; ++v) usk[v] = __ldg(ps + (size_t)v * NCELL);
@@ -887,7 +892,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
         const int base = yd ? 16 * 20 + r + 2 : (r + 2) * 20 + 16;
         const int stp = yd ? 20 : 1;
         const int fs = yd ? 1 : 0;
-        R* dstp = yd ? sFy + 16 * FP + r : sFx + S::xf(r, 16);
+        R* dstp = yd ? sFy + S::yf(16, r) : sFx + S::xf(r, 16);
         const int ns = yd ? FYN : FXN;
         R pl[NV], pr[NV];
         if constexpr (SHARED_SLOPES) {
@@ -945,9 +950,8 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
     {
       const size_t cell = (size_t)k * 256 + cell2;
       const size_t base = (size_t)b * NT * NCELL + cell;
-      // U_s of the cell: the raw TMA slot, or global memory (layout with three slots)
-      const R* raw = US_GLOBAL ? Us + base : sRaw + (size_t)((k - k0 + 2) % RAW) * NT * 256 + cell2;
-      constexpr int RSTR = US_GLOBAL ? NCELL : 256;
+      // U_s of the cell: the raw TMA slot, or loaded above
+      const R* raw = sRaw + (size_t)((k - k0 + 2) % RAW) * NT * 256 + cell2;
       R out[NV];
       if constexpr (P::SOURCE) {
         // all flux divergences first: the source needs those of other variables
@@ -968,7 +972,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
         if constexpr (P::QV >= 0) L[P::QV] = (htc_g - pc[P::QV]) * rq4;   // -(q - target) / tau
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
-          R val = raw[(size_t)v * RSTR];
+          R val = US_GLOBAL ? usk[US_GLOBAL ? v : 0] : raw[v * 256];
           if (v < P::FROZEN) {
             val = val + rdt * L[v];
             if (combine) val = ra * unk[v] + rb * val;
@@ -986,7 +990,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
             if (v >= P::BOFF && v < P::BOFF + 3) L = L + rsrc[v - P::BOFF];
             if (v == P::IE) L = L + rsrc[3];
           }
-          R val = (PRIMIN ? usk[PRIMIN ? v : 0] : raw[(size_t)v * RSTR]) + rdt * L;
+          R val = (US_GLOBAL ? usk[US_GLOBAL ? v : 0] : raw[v * 256]) + rdt * L;
           if (combine) val = ra * unk[v] + rb * val;
           out[v] = val;
           fzd[v] = fzu[v];

@@ -84,23 +84,25 @@ static cudaError_t stage_go_layout(const StageArgs& a, cudaStream_t s) {
 
 // Staging layouts: STAGE_LAYOUT_RING4 = four raw slots, one flux buffer, two barriers per
 // plane; STAGE_LAYOUT_RING5_DB = five raw slots, two flux buffers, one barrier per plane;
-// STAGE_LAYOUT_RING3_DB = three raw slots, two flux buffers, one barrier per plane, the update
-// reading its stage input from global memory (L2) instead of a raw slot. The default (layout
-// 0) takes layout 2 where it keeps as many CTAs per SM as layout 1, else layout 1 (FP32
-// stencils; FP64 keeps layout 1). Layout 3 is an autotuner choice: at equal CTAs per SM its
-// global re-read of U_s costs about what its saved barrier gains (MHD 0.870 against 0.860 ms,
-// FFHD 0.459 against 0.450 ms per 256^3 stage launch). Only the default layout cuts blocks along
-// z (stage_zsplit).
+// STAGE_LAYOUT_RING3_DB = three raw slots, two flux buffers, one barrier per plane, the update's
+// stage input loaded from global memory (L2) ahead of the face work instead of kept in a raw
+// slot. The default (layout 0) takes layout 2 where it keeps as many CTAs per SM as layout 1, else
+// layout 3 where that keeps two (256^3 MHD launch: layout 1 858 us, layout 3 831; with resistivity
+// on 1728 blocks 396 and 388), else layout 1: three CTAs per SM cover the second barrier as well
+// as layout 3 saves it (FFHD, 1728 blocks: 195 us either way). FP64 keeps layout 1. Only the
+// default layout cuts blocks along z (stage_zsplit).
 template <template <typename> class PT, typename R, int LIM, int FLUX>
 static cudaError_t stage_go(const StageArgs& a, cudaStream_t s) {
   if constexpr (sizeof(R) == 8) {
     return stage_go_layout<PT, R, LIM, FLUX, 4, 1, true>(a, s);
   } else {
-    constexpr int dflt = stage_minb<PT, R, 5, 2>() >= stage_minb<PT, R, 4, 1>() ? STAGE_LAYOUT_RING5_DB
-                                                                                 : STAGE_LAYOUT_RING4;
+    constexpr int m1 = stage_minb<PT, R, 4, 1>();
+    constexpr int dflt = stage_minb<PT, R, 5, 2>() >= m1             ? STAGE_LAYOUT_RING5_DB
+                         : m1 == 2 && stage_minb<PT, R, 3, 2>() == 2 ? STAGE_LAYOUT_RING3_DB
+                                                                     : STAGE_LAYOUT_RING4;
     const int lay = a.layout == 0 ? dflt : a.layout;
     if (lay == STAGE_LAYOUT_RING5_DB) return stage_go_layout<PT, R, LIM, FLUX, 5, 2, dflt == STAGE_LAYOUT_RING5_DB>(a, s);
-    if (lay == STAGE_LAYOUT_RING3_DB) return stage_go_layout<PT, R, LIM, FLUX, 3, 2, false>(a, s);
+    if (lay == STAGE_LAYOUT_RING3_DB) return stage_go_layout<PT, R, LIM, FLUX, 3, 2, dflt == STAGE_LAYOUT_RING3_DB>(a, s);
     return stage_go_layout<PT, R, LIM, FLUX, 4, 1, dflt == STAGE_LAYOUT_RING4>(a, s);
   }
 }
