@@ -361,12 +361,14 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   constexpr bool US_GLOBAL = RAW == 3 || PRIMIN;   // the update reads U_s of its cell from global memory
   using S = StageSmem<PT, R, RAW, SFB>;
   constexpr int NV = P::NV, NA = P::NA, NT = NV + NA;
-  // FP32 with HLL or TVDLF: x- and y-faces solved as packed pairs
-  constexpr bool PAIRED = sizeof(R) == 4 && PairPhys<P>::OK && (FLUX == FLUX_HLL || FLUX == FLUX_TVDLF);
+  // FP32: x- and y-faces solved as packed pairs, z-faces left with right (not HLLC, which picks
+  // one of the sides)
+  constexpr bool PAIRED = sizeof(R) == 4 && PairPhys<P>::OK;
+  constexpr bool PAIRED_Z = PAIRED && FLUX != FLUX_HLLC;
   constexpr int NAW = NA > 0 ? NA : 1;
   constexpr bool RESP = res_of<P>::value;   // resistive MHD sources
   constexpr R FU = R(flux_unit<FLUX>());    // unit of the scalar solver's fluxes
-  constexpr R FUZ = PAIRED ? R(1) : FU;     // unit of the z-face fluxes
+  constexpr R FUZ = PAIRED_Z ? R(1) : FU;     // unit of the z-face fluxes
   // FP64: the x/y slopes of a plane are formed once per cell and shared through the flux
   // buffers (below; three more CTA barriers per plane), instead of by the faces on both sides.
   // The FP64 units bind (86% busy at 8% of the issue slots): with the comparisons and roots
@@ -643,7 +645,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
       pr[v] = c[v] - h;
       hz[v] = h;
     }
-    if constexpr (PAIRED) riemann_z_lr<P, FLUX>(pl, pr, f, pp);
+    if constexpr (PAIRED_Z) riemann_z_lr<P, FLUX>(pl, pr, f, pp);
     else riemann<P, R, 2, FLUX>(pl, pr, f, pp);
   };
   // States of the face between cells q[o] and q[2 o] of a ring plane (o: the step along the

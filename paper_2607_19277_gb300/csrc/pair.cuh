@@ -331,11 +331,43 @@ __host__ __device__ constexpr bool glm_var(int v) {
   return P::GLM && (v == P::BOFF || v == P::NV - 1);
 }
 
-// HLL or TVDLF flux of the pair from reconstructed primitive states (modified in place).
+// HLL, TVDLF or (HD) HLLC flux of the pair from reconstructed primitive states (modified in place).
 template <class P, int FLUX>
 __device__ __forceinline__ void riemann2(f2* pl, f2* pr, f2* f, const PairK& k) {
   using Q = PairPhys<P>;
   constexpr int NV = Q::NV;
+  if constexpr (FLUX == FLUX_HLLC) {   // the scalar solver's HLLC, the side chosen per half
+    f2 lml, lpl, lmr, lpr;
+    Q::lambdas(pl, lml, lpl, k);
+    Q::lambdas(pr, lmr, lpr, k);
+    const f2 sl = min2(lml, lmr), sr = max2(lpl, lpr);
+    const f2 ml = pl[0] * (sl - pl[1]), mr = pr[0] * (sr - pr[1]);
+    const f2 ss = ((pr[4] - pl[4]) + (ml * pl[1] - mr * pr[1])) * rcp2(ml - mr);
+    float sx, sy;
+    f2_split(ss, sx, sy);
+    const bool lx = sx >= 0.0f, ly = sy >= 0.0f;
+    auto pick = [&](f2 l, f2 r) {
+      float ax, ay, bx, by;
+      f2_split(l, ax, ay);
+      f2_split(r, bx, by);
+      return f2_of(lx ? ax : bx, ly ? ay : by);
+    };
+    f2 q[NV], u[NV], fk[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) q[v] = pick(pl[v], pr[v]);
+    const f2 sk = pick(sl, sr), mk = pick(ml, mr);
+    const f2 s = pick(min2(sl, k.zero), max2(sr, k.zero));
+    Q::prim2cons(q, u, k);
+    Q::flux(q, u, fk, k);
+    const f2 fac = mk * rcp2(sk - ss);
+    const f2 us4 = fac * fma2(ss - q[1], fma2(q[4], rcp2(mk), ss), u[4] * rcp2(q[0]));
+    f[0] = fma2(s, fac - u[0], fk[0]);
+    f[1] = fma2(s, fac * ss - u[1], fk[1]);
+    f[2] = fma2(s, fac * q[2] - u[2], fk[2]);
+    f[3] = fma2(s, fac * q[3] - u[3], fk[3]);
+    f[4] = fma2(s, us4 - u[4], fk[4]);
+    return;
+  }
   Q::interface(pl, pr, k);
   f2 ul[NV], ur[NV], fl[NV], fr[NV];
   Q::prim2cons(pl, ul, k);
