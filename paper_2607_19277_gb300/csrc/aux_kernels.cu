@@ -243,7 +243,10 @@ __global__ void __launch_bounds__(256) speeds_kernel(const R* __restrict__ U,
   constexpr int NV = P::NV, NA = P::NA, NT = NV + NA;
   chain_wait();
   const int b = wl ? wl[blockIdx.x] : (int)blockIdx.x;
-  const R dxr[3] = {R(bd[b].dx[0]), R(bd[b].dx[1]), R(bd[b].dx[2])};
+  __shared__ R s_id[3];
+  if (threadIdx.x < 3) s_id[threadIdx.x] = R(1.0 / bd[b].dx[threadIdx.x]);
+  __syncthreads();
+  const R id[3] = {s_id[0], s_id[1], s_id[2]};
   R ssum = R(0), smax = R(0);
   int st = 0;
   const R* base = U + (size_t)b * NT * NCELL;
@@ -254,7 +257,7 @@ __global__ void __launch_bounds__(256) speeds_kernel(const R* __restrict__ U,
 #pragma unroll
     for (int v = 0; v < NV; ++v) u[v] = base[(size_t)v * NCELL + c];
     if constexpr (NA > 0) aux[0] = base[(size_t)NV * NCELL + c];
-    cell_speeds<PT, R>(u, aux, pp, dxr, ssum, smax, st);
+    cell_speeds<PT, R>(u, aux, pp, id, ssum, smax, st);
   }
   block_max2<256>(ssum, smax, speeds + 2 * (solve_of ? solve_of[b] : 0));
   if (st) atomicOr(status, st);
@@ -614,6 +617,8 @@ __global__ void __launch_bounds__(256) prim_pass_kernel(const R* __restrict__ U,
   R u[NT], p[NV], aux[NA > 0 ? NA : 1];
 #pragma unroll
   for (int v = 0; v < NT; ++v) u[v] = src[(size_t)v * vs];
+  __shared__ R s_id[3];
+  if (speeds && b >= 0 && threadIdx.x < 3) s_id[threadIdx.x] = R(1.0 / bd[b].dx[threadIdx.x]);
   if constexpr (NA > 0) {
 #pragma unroll
     for (int i = 0; i < NA; ++i) aux[i] = u[NV + i];
@@ -628,9 +633,10 @@ __global__ void __launch_bounds__(256) prim_pass_kernel(const R* __restrict__ U,
   for (int i = 0; i < NA; ++i) dst[(size_t)(NV + i) * vs] = aux[i];
   if (st) atomicOr(status, st);
   if (speeds && b >= 0) {             // CTA-uniform: a pool plane, not a ghost slot
-    const R dxr[3] = {R(bd[b].dx[0]), R(bd[b].dx[1]), R(bd[b].dx[2])};
+    __syncthreads();
+    const R id[3] = {s_id[0], s_id[1], s_id[2]};
     R ssum = R(0), smax = R(0);
-    prim_speeds<PT, R>(p, pp, dxr, ssum, smax);
+    prim_speeds<PT, R>(p, pp, id, ssum, smax);
     block_max2<256>(ssum, smax, speeds + 2 * (solve_of ? solve_of[b] : 0));
   }
 }

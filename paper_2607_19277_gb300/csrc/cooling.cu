@@ -158,7 +158,10 @@ __global__ void __launch_bounds__(256) cooling_kernel(R* __restrict__ U, const B
   const int sv = solve_of ? solve_of[b] : 0;
   const R dt = R(frac * dtch[2 * sv]);
   const R ig1 = pp.ig1;
-  const R dxr[3] = {R(bd[b].dx[0]), R(bd[b].dx[1]), R(bd[b].dx[2])};
+  __shared__ R s_id[3];
+  if (threadIdx.x < 3) s_id[threadIdx.x] = R(1.0 / bd[b].dx[threadIdx.x]);
+  __syncthreads();
+  const R id[3] = {s_id[0], s_id[1], s_id[2]};
   R ssum = R(0), smax = R(0);
   int st = 0;
   R* base = U + (size_t)b * NV * NCELL;
@@ -175,7 +178,7 @@ __global__ void __launch_bounds__(256) cooling_kernel(R* __restrict__ U, const B
     const R tn = cool_temperature<R>(rho, T, dt, c, seg);
     u[IE] = u[IE] - rho * (T - tn) * ig1;
     base[(size_t)IE * NCELL + i] = u[IE];
-    if (speeds) cell_speeds<PT, R>(u, aux, pp, dxr, ssum, smax, st);
+    if (speeds) cell_speeds<PT, R>(u, aux, pp, id, ssum, smax, st);
   }
   if (speeds) block_max2<256>(ssum, smax, speeds + 2 * sv);
   if (st) atomicOr(status, st);

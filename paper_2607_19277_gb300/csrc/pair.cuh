@@ -54,12 +54,6 @@ __device__ __forceinline__ f2 rcp2(f2 a) {
   f2_split(a, x, y);
   return f2_of(1.0f / x, 1.0f / y);
 }
-__device__ __forceinline__ f2 div2(f2 a, f2 b) {
-  float ax, ay, bx, by;
-  f2_split(a, ax, ay);
-  f2_split(b, bx, by);
-  return f2_of(ax / bx, ay / by);
-}
 __device__ __forceinline__ f2 sqrt2(f2 a) {
   float x, y;
   f2_split(a, x, y);
@@ -81,6 +75,13 @@ __device__ __forceinline__ f2 abs2(f2 a) {
   float x, y;
   f2_split(a, x, y);
   return f2_of(fabsf(x), fabsf(y));
+}
+
+__device__ __forceinline__ f2 add_abs2(f2 a, f2 b) {   // |a| + b
+  float ax, ay, bx, by;
+  f2_split(a, ax, ay);
+  f2_split(b, bx, by);
+  return f2_of(fabsf(ax) + bx, fabsf(ay) + by);
 }
 
 // Half limited slope of each half (the scalar half_slope's limiters).
@@ -156,10 +157,9 @@ struct PairPhys<HdPhys<float>> {
     f[3] = u[3] * vd;
     f[4] = vd * (u[4] + p[4]);
   }
-  __device__ static __forceinline__ void lambdas(const f2* p, f2& lm, f2& lp, const PairK& k) {
-    const f2 c = sqrt2(div2(k.gamma * p[4], p[0]));
-    lm = p[1] - c;
-    lp = p[1] + c;
+  __device__ static __forceinline__ void waves(const f2* p, f2& mid, f2& half, const PairK& k) {
+    mid = p[1];
+    half = sqrt2(k.gamma * p[4] * rcp2(p[0]));
   }
 };
 
@@ -209,15 +209,14 @@ struct PairPhys<MhdPhys<float>> {
     f[7] = fma2(vd, p[7], p[3] * nbd);
     f[8] = k.ch2 * p[5];
   }
-  __device__ static __forceinline__ void lambdas(const f2* p, f2& lm, f2& lp, const PairK& k) {
+  __device__ static __forceinline__ void waves(const f2* p, f2& mid, f2& half, const PairK& k) {
     const f2 ir = rcp2(p[0]);
     const f2 a2 = k.gamma * p[4] * ir;
     const f2 s = fma2(b2(p), ir, a2);
     const f2 bd2 = p[5] * p[5] * ir;
     const f2 disc = max2(fma2(s, s, k.m4 * a2 * bd2), k.zero);
-    const f2 cf = sqrt2(k.half * (s + sqrt2(disc)));
-    lm = p[1] - cf;
-    lp = p[1] + cf;
+    mid = p[1];
+    half = sqrt2(k.half * (s + sqrt2(disc)));
   }
 };
 
@@ -258,12 +257,9 @@ struct PairPhys<FfhdPhysT<float, HTC>> {
     for (int i = 3; i < NV; ++i) f[i] = k.zero;
     f[B] = b;
   }
-  __device__ static __forceinline__ void lambdas(const f2* p, f2& lm, f2& lp, const PairK& k) {
-    const f2 c = sqrt2(div2(k.gamma * p[2], p[0]));
-    const f2 a = p[1] * p[B];
-    const f2 w = c * abs2(p[B]);
-    lm = a - w;
-    lp = a + w;
+  __device__ static __forceinline__ void waves(const f2* p, f2& mid, f2& half, const PairK& k) {
+    mid = p[1] * p[B];
+    half = sqrt2(k.gamma * p[2] * rcp2(p[0])) * abs2(p[B]);
   }
 };
 
@@ -311,17 +307,15 @@ struct PairPhys<SrhdPhysE<float, EOS>> {
     f[3] = u[3] * vd;
     f[4] = u[1] - f[0];
   }
-  __device__ static __forceinline__ void lambdas(const f2* p, f2& lm, f2& lp, const PairK& k) {
+  // max |mid -+ half| (TVDLF, the only solver of the module)
+  __device__ static __forceinline__ f2 fastest(const f2* p, const PairK& k) {
     const f2 il = rcp2(gam(p, k));
     const f2 vd = p[1] * il;
     f2 w, cs2;
     closure(p, w, cs2, k);
     const f2 il2 = il * il;                       // 1 - v^2
     const f2 den = k.one - (k.one - il2) * cs2, a = vd * (k.one - cs2);
-    const f2 root = sqrt2(max2(cs2 * il2 * (den - vd * a), k.zero));
-    const f2 iden = rcp2(den);
-    lm = (a - root) * iden;
-    lp = (a + root) * iden;
+    return add_abs2(a, sqrt2(max2(cs2 * il2 * (den - vd * a), k.zero))) * rcp2(den);
   }
 };
 
@@ -331,16 +325,32 @@ __host__ __device__ constexpr bool glm_var(int v) {
   return P::GLM && (v == P::BOFF || v == P::NV - 1);
 }
 
+// Fastest speed max |mid -+ half| = |mid| + half of each half's state.
+template <class P>
+struct is_srhd : std::false_type {};
+template <typename R, int EOS>
+struct is_srhd<SrhdPhysE<R, EOS>> : std::true_type {};
+template <class P>
+__device__ __forceinline__ f2 fastest(const f2* p, const PairK& k) {
+  if constexpr (is_srhd<P>::value) {
+    return PairPhys<P>::fastest(p, k);
+  } else {
+    f2 mid, half;
+    PairPhys<P>::waves(p, mid, half, k);
+    return add_abs2(mid, half);
+  }
+}
+
 // HLL, TVDLF or (HD) HLLC flux of the pair from reconstructed primitive states (modified in place).
 template <class P, int FLUX>
 __device__ __forceinline__ void riemann2(f2* pl, f2* pr, f2* f, const PairK& k) {
   using Q = PairPhys<P>;
   constexpr int NV = Q::NV;
   if constexpr (FLUX == FLUX_HLLC) {   // the scalar solver's HLLC, the side chosen per half
-    f2 lml, lpl, lmr, lpr;
-    Q::lambdas(pl, lml, lpl, k);
-    Q::lambdas(pr, lmr, lpr, k);
-    const f2 sl = min2(lml, lmr), sr = max2(lpl, lpr);
+    f2 vml, vhl, vmr, vhr;
+    Q::waves(pl, vml, vhl, k);
+    Q::waves(pr, vmr, vhr, k);
+    const f2 sl = min2(vml - vhl, vmr - vhr), sr = max2(vml + vhl, vmr + vhr);
     const f2 ml = pl[0] * (sl - pl[1]), mr = pr[0] * (sr - pr[1]);
     const f2 ss = ((pr[4] - pl[4]) + (ml * pl[1] - mr * pr[1])) * rcp2(ml - mr);
     float sx, sy;
@@ -374,11 +384,8 @@ __device__ __forceinline__ void riemann2(f2* pl, f2* pr, f2* f, const PairK& k) 
   Q::prim2cons(pr, ur, k);
   Q::flux(pl, ul, fl, k);
   Q::flux(pr, ur, fr, k);
-  f2 lml, lpl, lmr, lpr;
-  Q::lambdas(pl, lml, lpl, k);
-  Q::lambdas(pr, lmr, lpr, k);
   if constexpr (FLUX == FLUX_TVDLF) {
-    const f2 c = max2(max2(abs2(lml), abs2(lpl)), max2(abs2(lmr), abs2(lpr)));
+    const f2 c = max2(fastest<P>(pl, k), fastest<P>(pr, k));
     const f2 nhc = k.zero - k.half * c;
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
@@ -388,8 +395,11 @@ __device__ __forceinline__ void riemann2(f2* pl, f2* pr, f2* f, const PairK& k) 
       else f[v] = fma2(nhc, ur[v] - ul[v], k.half * (fl[v] + fr[v]));
     }
   } else {
-    const f2 sl = min2(min2(lml, lmr), k.zero);
-    const f2 sr = max2(max2(lpl, lpr), k.zero);
+    f2 vml, vhl, vmr, vhr;   // middle and half width of each side's speeds
+    Q::waves(pl, vml, vhl, k);
+    Q::waves(pr, vmr, vhr, k);
+    const f2 sl = min2(min2(vml - vhl, vmr - vhr), k.zero);
+    const f2 sr = max2(max2(vml + vhl, vmr + vhr), k.zero);
     const f2 inv = rcp2(sr - sl);
     const f2 wl = sr * inv, nwr = (k.zero - sl) * inv, wd = sl * wl;
 #pragma unroll
@@ -415,17 +425,19 @@ __device__ __forceinline__ void riemann_z_lr(float* pl, float* pr, float* f, con
   for (int v = 0; v < NV; ++v) q[v] = f2_of(pl[Q::zrot(v)], pr[Q::zrot(v)]);
   Q::prim2cons(q, u, k);
   Q::flux(q, u, fq, k);
-  f2 lm, lp;
-  Q::lambdas(q, lm, lp, k);
-  float lml, lmr, lpl, lpr;
-  f2_split(lm, lml, lmr);
-  f2_split(lp, lpl, lpr);
   f2 w, dw;   // F = w.x fl + w.y fr + dw.x ul + dw.y ur
   if constexpr (FLUX == FLUX_TVDLF) {
-    const float c = fmaxf(fmaxf(fabsf(lml), fabsf(lpl)), fmaxf(fabsf(lmr), fabsf(lpr)));
+    float cl, cr;
+    f2_split(fastest<P>(q, k), cl, cr);
+    const float c = fmaxf(cl, cr);
     w = k.half;
     dw = f2_of(0.5f * c, -0.5f * c);
   } else {
+    f2 mid, half;
+    Q::waves(q, mid, half, k);
+    float lml, lmr, lpl, lpr;
+    f2_split(mid - half, lml, lmr);
+    f2_split(mid + half, lpl, lpr);
     const float sl = fminf(fminf(lml, lmr), 0.0f);
     const float sr = fmaxf(fmaxf(lpl, lpr), 0.0f);
     const float inv = 1.0f / (sr - sl);

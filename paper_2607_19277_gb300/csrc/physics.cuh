@@ -170,7 +170,7 @@ struct HdPhys {
     p[1] = vx;
     p[2] = vy;
     p[3] = vz;
-    p[4] = g1 * (u[4] - R(0.5) * rho * (vx * vx + vy * vy + vz * vz));
+    p[4] = g1 * (u[4] - R(0.5) * (u[1] * vx + u[2] * vy + u[3] * vz));
     st |= (!rpos(rho) | !rpos(p[4])) ? ST_EUNPHYS : 0;
   }
 
@@ -183,9 +183,9 @@ struct HdPhys {
     u[4] = p[4] * ig1 + R(0.5) * p[0] * (p[1] * p[1] + p[2] * p[2] + p[3] * p[3]);
   }
 
-  // Conserved state, flux along D and slowest / fastest speed of a face state.
+  // Conserved state, flux along D and the interval mid -+ half of the speeds of a face state.
   template <int D>
-  __device__ static __forceinline__ void side(const R* p, R* u, R* f, R& lm, R& lp, const PhysParamsT<R>& pp) {
+  __device__ static __forceinline__ void side(const R* p, R* u, R* f, R& mid, R& half, const PhysParamsT<R>& pp) {
     const R vd = p[1 + D];
     u[0] = p[0];
     u[1] = p[0] * p[1];
@@ -198,14 +198,13 @@ struct HdPhys {
     f[3] = u[3] * vd;
     f[1 + D] = u[1 + D] * vd + p[4];
     f[4] = vd * (u[4] + p[4]);
-    lambdas<D>(p, lm, lp, pp);
+    waves<D>(p, mid, half, pp);
   }
 
   template <int D>
-  __device__ static __forceinline__ void lambdas(const R* p, R& lm, R& lp, const PhysParamsT<R>& pp) {
-    const R c = rsqrt_(rdiv(pp.gamma * p[4], p[0]));
-    lm = p[1 + D] - c;
-    lp = p[1 + D] + c;
+  __device__ static __forceinline__ void waves(const R* p, R& mid, R& half, const PhysParamsT<R>& pp) {
+    mid = p[1 + D];
+    half = rsqrt_(rdiv(pp.gamma * p[4], p[0]));
   }
 
   template <int D>
@@ -237,7 +236,8 @@ struct MhdPhys {
     p[1] = vx;
     p[2] = vy;
     p[3] = vz;
-    p[4] = g1 * (u[4] - R(0.5) * rho * (vx * vx + vy * vy + vz * vz) - R(0.5) * b2);
+    if constexpr (sizeof(R) == 8) p[4] = g1 * (u[4] - R(0.5) * ((u[1] * vx + u[2] * vy + u[3] * vz) + b2));
+    else p[4] = g1 * (u[4] - R(0.5) * rho * (vx * vx + vy * vy + vz * vz) - R(0.5) * b2);
     p[5] = u[5];
     p[6] = u[6];
     p[7] = u[7];
@@ -260,11 +260,11 @@ struct MhdPhys {
   }
 
   // Conserved state, flux along D (without those of B_d and psi, which riemann sets from the
-  // face values) and slowest / fastest speed of a face state. FP64: the fast speed from
+  // face values) and the interval of the speeds of a face state. FP64: the fast speed from
   // S = gamma p + B^2, cf^2 = (S + sqrt(S^2 - 4 gamma p B_d^2)) / (2 rho), which divides by the
   // density once; FP32 keeps every square near a^4, whose range it can hold.
   template <int D>
-  __device__ static __forceinline__ void side(const R* p, R* u, R* f, R& lm, R& lp, const PhysParamsT<R>& pp) {
+  __device__ static __forceinline__ void side(const R* p, R* u, R* f, R& mid, R& half, const PhysParamsT<R>& pp) {
     const R vd = p[1 + D], bd = p[5 + D];
     const R b2 = p[5] * p[5] + p[6] * p[6] + p[7] * p[7];
     const R vb = p[1] * p[5] + p[2] * p[6] + p[3] * p[7];
@@ -293,25 +293,23 @@ struct MhdPhys {
       const R gp = pp.gamma * p[4];
       const R s = gp + b2;
       const R disc = rmax(s * s - (R(4) * gp) * (bd * bd), R(0));
-      const R cf = rsqrt_((R(0.5) * (s + rsqrt_(disc))) * rrcp(p[0]));
-      lm = vd - cf;
-      lp = vd + cf;
+      mid = vd;
+      half = rsqrt_((R(0.5) * (s + rsqrt_(disc))) * rrcp(p[0]));
     } else {
-      lambdas<D>(p, lm, lp, pp);
+      waves<D>(p, mid, half, pp);
     }
   }
 
   template <int D>
-  __device__ static __forceinline__ void lambdas(const R* p, R& lm, R& lp, const PhysParamsT<R>& pp) {
+  __device__ static __forceinline__ void waves(const R* p, R& mid, R& half, const PhysParamsT<R>& pp) {
     const R ir = rrcp(p[0]);
     const R a2 = pp.gamma * p[4] * ir;
     const R b2 = (p[5] * p[5] + p[6] * p[6] + p[7] * p[7]) * ir;
     const R bd2 = p[5 + D] * p[5 + D] * ir;
     const R s = a2 + b2;
     const R disc = rmax(s * s - R(4) * a2 * bd2, R(0));
-    const R cf = rsqrt_(R(0.5) * (s + rsqrt_(disc)));
-    lm = p[1 + D] - cf;
-    lp = p[1 + D] + cf;
+    mid = p[1 + D];
+    half = rsqrt_(R(0.5) * (s + rsqrt_(disc)));
   }
 
   // Exact solution of the linear (B_d, psi) subsystem at the face (Dedner et al. 2002):
@@ -671,26 +669,18 @@ struct SrhdPhysE {
     u[4] = lor * lrh - p[4] - lr;
   }
 
-  // Conserved state, flux along D and slowest / fastest speed of a face state: one root and one
+  // Conserved state, flux along D and the interval of the speeds of a face state: one root and one
   // quotient for Gamma, rho h = rho + gamma/(gamma-1) p without a quotient (ideal gas), the two
   // factors of the speeds' root under one root: three quotients and two roots where formulas
   // taken one by one need six and four. Quotients and roots are most of these kernels' work:
   // a 48x64x80 FP64 solve took 6.56 -> 5.45 ms, a batch of 12 FP32 solves 10.9 -> 10.2 ms.
   template <int D>
-  __device__ static __forceinline__ void side(const R* p, R* u, R* f, R& lm, R& lp, const PhysParamsT<R>& pp) {
+  __device__ static __forceinline__ void side(const R* p, R* u, R* f, R& mid, R& half, const PhysParamsT<R>& pp) {
     const R lor = rsqrt_(R(1) + p[1] * p[1] + p[2] * p[2] + p[3] * p[3]);
     const R il = rrcp(lor);
     const R vd = p[1 + D] * il;
-    R w, cs2;                                   // rho h, squared sound speed
-    if constexpr (EOS == EOS_SYNGE) {
-      const R th = p[4] * rrcp(p[0]);
-      const R h = Eos::enthalpy(th, pp);
-      w = p[0] * h;
-      cs2 = Eos::sound_speed2(th, h, pp);
-    } else {
-      w = p[0] + pp.gg1 * p[4];
-      cs2 = (pp.gamma * p[4]) * rrcp(w);
-    }
+    R w, cs2;
+    closure(p, w, cs2, pp);
     const R lr = lor * p[0], lw = lor * w;
     u[0] = lr;
     u[1] = lw * p[1];
@@ -703,33 +693,37 @@ struct SrhdPhysE {
     f[3] = u[3] * vd;
     f[1 + D] += p[4];
     f[4] = u[1 + D] - f[0];
+    speeds_of(vd, il, cs2, mid, half);
+  }
+
+  // rho h and the squared sound speed
+  __device__ static __forceinline__ void closure(const R* p, R& w, R& cs2, const PhysParamsT<R>& pp) {
+    if constexpr (EOS == EOS_SYNGE) {
+      const R th = p[4] * rrcp(p[0]);
+      const R h = Eos::enthalpy(th, pp);
+      w = p[0] * h;
+      cs2 = Eos::sound_speed2(th, h, pp);
+    } else {
+      w = p[0] + pp.gg1 * p[4];
+      cs2 = (pp.gamma * p[4]) * rrcp(w);
+    }
+  }
+  // Middle and half width of the interval of characteristic speeds along a direction with velocity
+  // vd, il = 1 / Gamma.
+  __device__ static __forceinline__ void speeds_of(R vd, R il, R cs2, R& mid, R& half) {
     const R il2 = il * il;                      // 1 - v^2
     const R den = R(1) - (R(1) - il2) * cs2, a = vd * (R(1) - cs2);
-    const R root = rsqrt_(rmax((cs2 * il2) * (den - vd * a), R(0)));
     const R iden = rrcp(den);
-    lm = (a - root) * iden;
-    lp = (a + root) * iden;
+    mid = a * iden;
+    half = rsqrt_(rmax((cs2 * il2) * (den - vd * a), R(0))) * iden;
   }
 
   template <int D>
-  __device__ static __forceinline__ void lambdas(const R* p, R& lm, R& lp, const PhysParamsT<R>& pp) {
-    const R lor2 = R(1) + p[1] * p[1] + p[2] * p[2] + p[3] * p[3];
-    const R v2 = R(1) - rrcp(lor2);
-    const R vd = rdiv(p[1 + D], rsqrt_(lor2));
-    R cs2;
-    if constexpr (EOS == EOS_SYNGE) {
-      const R th = rdiv(p[4], p[0]);
-      cs2 = Eos::sound_speed2(th, Eos::enthalpy(th, pp), pp);
-    } else {
-      const R h = R(1) + rdiv(pp.gg1 * p[4], p[0]);
-      cs2 = rdiv(pp.gamma * p[4], p[0] * h);
-    }
-    const R cs = rsqrt_(cs2);
-    const R den = R(1) - v2 * cs2;
-    const R root = cs * rsqrt_(rmax((R(1) - v2) * (R(1) - v2 * cs2 - vd * vd * (R(1) - cs2)), R(0)));
-    const R iden = rrcp(den);
-    lm = (vd * (R(1) - cs2) - root) * iden;
-    lp = (vd * (R(1) - cs2) + root) * iden;
+  __device__ static __forceinline__ void waves(const R* p, R& mid, R& half, const PhysParamsT<R>& pp) {
+    const R il = rrcp(rsqrt_(R(1) + p[1] * p[1] + p[2] * p[2] + p[3] * p[3]));
+    R w, cs2;
+    closure(p, w, cs2, pp);
+    speeds_of(p[1 + D] * il, il, cs2, mid, half);
   }
 
   template <int D>
@@ -783,11 +777,11 @@ struct FfhdPhysT {
     for (int i = 3; i < NV; ++i) u[i] = p[i];
   }
 
-  // Conserved state, flux along D and slowest / fastest speed of a face state.
+  // Conserved state, flux along D and the interval mid -+ half of the speeds of a face state.
   template <int D>
-  __device__ static __forceinline__ void side(const R* p, R* u, R* f, R& lm, R& lp, const PhysParamsT<R>& pp) {
+  __device__ static __forceinline__ void side(const R* p, R* u, R* f, R& mid, R& half, const PhysParamsT<R>& pp) {
     prim2cons(p, u, pp);
-    lambdas<D>(p, lm, lp, pp);
+    waves<D>(p, mid, half, pp);
     const R b = p[BOFF + D];
     const R vb = p[1] * b;
     f[0] = u[0] * vb;
@@ -800,13 +794,11 @@ struct FfhdPhysT {
   }
 
   template <int D>
-  __device__ static __forceinline__ void lambdas(const R* p, R& lm, R& lp, const PhysParamsT<R>& pp) {
+  __device__ static __forceinline__ void waves(const R* p, R& mid, R& half, const PhysParamsT<R>& pp) {
     const R c = rsqrt_(rdiv(pp.gamma * p[2], p[0]));
     const R b = p[BOFF + D];
-    const R a = p[1] * b;
-    const R w = c * rabs(b);
-    lm = a - w;
-    lp = a + w;
+    mid = p[1] * b;
+    half = c * rabs(b);
   }
 
   template <int D>
@@ -837,7 +829,7 @@ __host__ __device__ constexpr double flux_unit() {
 template <class P, typename R, int D, int FLUX>
 __device__ __forceinline__ void riemann(R* pl, R* pr, R* f, const PhysParamsT<R>& pp) {
   constexpr int NV = P::NV;
-  R lml, lpl, lmr, lpr;
+  R vml, vhl, vmr, vhr;   // middle and half width of each side's speeds
   if constexpr (FLUX == FLUX_HLLC) {
     // HLLC (Toro, Spruce & Speares 1994) for hydrodynamics: the HLL fan with the contact restored.
     // The contact speed S* tells the side K whose flux F_K + S (U*_K - U_K) the face has, S the
@@ -846,9 +838,9 @@ __device__ __forceinline__ void riemann(R* pl, R* pr, R* f, const PhysParamsT<R>
     // p_K/(rho_K (S_K - u_K)))]. The side is chosen before its conserved state, flux and star
     // state are formed, so these are formed once (210 FP64 blocks 1206 -> 992 us a launch, 1728
     // FP32 blocks 256 -> 234, in packed pairs 224).
-    P::template lambdas<D>(pl, lml, lpl, pp);
-    P::template lambdas<D>(pr, lmr, lpr, pp);
-    const R sl = rmin(lml, lmr), sr = rmax(lpl, lpr);
+    P::template waves<D>(pl, vml, vhl, pp);
+    P::template waves<D>(pr, vmr, vhr, pp);
+    const R sl = rmin(vml - vhl, vmr - vhr), sr = rmax(vml + vhl, vmr + vhr);
     const R vl = pl[1 + D], vr = pr[1 + D];
     const R ml = pl[0] * (sl - vl), mr = pr[0] * (sr - vr);
     const R ss = rdiv(pr[4] - pl[4] + ml * vl - mr * vr, ml - mr);
@@ -871,10 +863,10 @@ __device__ __forceinline__ void riemann(R* pl, R* pr, R* f, const PhysParamsT<R>
   }
   P::template interface<D>(pl, pr, pp);
   R ul[NV], ur[NV], fl[NV], fr[NV];
-  P::template side<D>(pl, ul, fl, lml, lpl, pp);
-  P::template side<D>(pr, ur, fr, lmr, lpr, pp);
+  P::template side<D>(pl, ul, fl, vml, vhl, pp);
+  P::template side<D>(pr, ur, fr, vmr, vhr, pp);
   if constexpr (FLUX == FLUX_TVDLF) {
-    const R c = rmax(rmax(rabs(lml), rabs(lpl)), rmax(rabs(lmr), rabs(lpr)));
+    const R c = rmax(rabs(vml) + vhl, rabs(vmr) + vhr);   // max |mid -+ half| = |mid| + half
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       if (v >= P::FROZEN) f[v] = fl[v] + fl[v];   // frozen variables: exact flux, no dissipation
@@ -882,8 +874,8 @@ __device__ __forceinline__ void riemann(R* pl, R* pr, R* f, const PhysParamsT<R>
       else f[v] = (fl[v] + fr[v]) - c * (ur[v] - ul[v]);
     }
   } else {
-    const R sl = rmin(rmin(lml, lmr), R(0));
-    const R sr = rmax(rmax(lpl, lpr), R(0));
+    const R sl = rmin(rmin(vml - vhl, vmr - vhr), R(0));
+    const R sr = rmax(rmax(vml + vhl, vmr + vhr), R(0));
     const R inv = rrcp(sr - sl);
     const R wl = sr * inv, wr = sl * inv, wd = sl * wl;
 #pragma unroll
