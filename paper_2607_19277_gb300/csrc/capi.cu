@@ -46,7 +46,8 @@ struct agile_mesh {
   int* d_status = nullptr;
   unsigned long long* d_speeds = nullptr;
   double* d_dtch = nullptr;
-  int* d_work = nullptr;            // per-stage block counters of the persistent launches
+  int* d_work = nullptr;            // per-stage item counters of the persistent launches
+  StageCut cut;                     // work items of the stage launches (stage_go)
   int* d_vars = nullptr;
   double* d_weights = nullptr;
   bool speeds_valid = false;
@@ -773,6 +774,7 @@ agile_status agile_step(agile_mesh* m, double dt) {
     A.tmap = &m->tmap[st == 0 ? 0 : st];
     A.solve_of = nullptr;
     A.work = m->d_work + st;
+    A.cut_cache = &m->cut;
     cudaEvent_t e0 = phase_begin(m);
     if (m->W) {                      // one recovery per stored cell, read by the stage kernel
       AuxArgs pa = aux_args(m, Us);
@@ -1188,6 +1190,7 @@ struct agile_batch {
   int grid = 0;                     // persistent CTAs of the stage launches (0: default)
   bool dynamic = true;              // blocks taken from an atomic counter (else strided)
   int layout = 0;                   // staging layout of the stage kernel (0: the default)
+  StageCut cut;                     // work items of the stage launches (stage_go)
   // refinement: ghost slots, flux registers and their tasks of all solves (indices offset)
   void* G = nullptr;
   void* FR = nullptr;
@@ -1839,6 +1842,7 @@ agile_status batch_enqueue_step(agile_batch* B) {
     A.work = B->dynamic ? B->d_work + st : nullptr;
     A.grid = B->grid;
     A.layout = B->layout;
+    A.cut_cache = &B->cut;
     if (B->W) {                       // one recovery per stored cell, read by the stage kernel
       AuxArgs pa = batch_aux(B, Us);
       if (st == 0) BCK(B, cudaMemsetAsync(B->d_speeds, 0, 2 * sizeof(unsigned long long) * B->nsolve, B->stream));
@@ -1904,6 +1908,7 @@ agile_status batch_stage1(agile_batch* B, int grid, bool dynamic, int layout) {
   A.work = dynamic ? B->d_work : nullptr;
   A.grid = grid;
   A.layout = layout;
+  A.cut_cache = &B->cut;
   if (B->W) {
     AuxArgs pa = batch_aux(B, B->U[0]);
     BCK(B, launch_prim_pass(pa, B->W, B->WG, B->nslots, nullptr, B->stream));

@@ -21,6 +21,36 @@ namespace agile {
 
 enum : int { STAGE_LAYOUT_RING4 = 1, STAGE_LAYOUT_RING5_DB = 2, STAGE_LAYOUT_RING3_DB = 3 };
 
+// Work items of a launch over nblk blocks: the first n1 blocks whole, of the others m items of a
+// planes each, then (behind all of those) one of the 16 - m a planes left, if any. Sizes fall
+// along the list, so that CTAs taking the next free item end close together.
+struct StageCut {
+  int nblk = -1;
+  int n1 = 0, a = NB, m = 1;
+  unsigned long long inv_m = 1ull << 32;   // ceil(2^32 / m): exact for items below 2^28
+  __host__ __device__ int rest() const { return NB - m * a; }
+  __host__ __device__ int items() const { return n1 + (nblk - n1) * (rest() > 0 ? m + 1 : m); }
+  __host__ __device__ bool whole() const { return n1 == nblk || a == NB; }
+  // block (index into the work list), first plane and planes of item w
+  __host__ __device__ void item(int w, int& blk, int& k0, int& nz) const {
+    const int nr = nblk - n1;
+    if (w < n1) {
+      blk = w;
+      k0 = 0;
+      nz = NB;
+    } else if (w - n1 < nr * m) {
+      const int v = w - n1, q = (int)((unsigned long long)(unsigned)v * inv_m >> 32);   // v / m
+      blk = n1 + q;
+      k0 = (v - q * m) * a;
+      nz = a;
+    } else {
+      blk = n1 + (w - n1 - nr * m);
+      k0 = m * a;
+      nz = rest();
+    }
+  }
+};
+
 struct StageArgs {
   const void* Us;           // stage input state (with aux)
   const void* Un;           // U^n for the combine (a != 0)
@@ -56,7 +86,8 @@ struct StageArgs {
   PhysParamsT<float> ppf;
   float fa = 0.0f, fb = 0.0f;
   int combine = 0;
-  int zs = 0;                   // a work item is 16 >> zs planes of a block (stage_go's rule)
+  StageCut cut;                 // the launch's work items, set by stage_go
+  StageCut* cut_cache = nullptr;  // host: the caller's copy, formed again when nblk changes
 };
 
 // Conserved + auxiliary values of the cell (x, y, z) of block b in the halo view: the
@@ -350,7 +381,7 @@ struct StageSmem {
 //   D. flux divergence, SSPRK combine and store of cell (x, y, k);
 //   -- CTA barrier, with one flux buffer only: the next plane's faces overwrite it --
 // Raw planes arrive by TMA one or two planes ahead of their conversion. With Z_CUT the launch's
-// work items are parts of blocks (A.zs): the same planes, faces and cells, the same arithmetic.
+// work items are parts of blocks (A.cut): the same planes, faces and cells, the same arithmetic.
 template <template <typename> class PT, typename R, int LIM, int FLUX, int MINB, int RAW, int SFB, bool Z_CUT>
 __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant__ CUtensorMap tmap,
                                                            StageArgs A) {
@@ -378,13 +409,11 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   // 0.96 ms per stage and a 128^3 MHD one from 5.5 to 4.6 ms. FP32 kernels are bound by
   // instruction issue and barriers, and form them twice.
   constexpr bool SHARED_SLOPES = sizeof(R) == 8;
-  // A work item is planes k0 .. k0 + nz - 1 of a block (the whole block for zs = 0): it reads
+  // A work item is planes k0 .. k0 + nz - 1 of a block (without Z_CUT the whole block): it reads
   // planes k0 - 2 .. k0 + nz + 1, TMA sequence 0 .. nz + 3.
-  const int zs = Z_CUT ? A.zs : 0;
-  const int nz = NB >> zs;
-  const int nitem = A.nblk << zs;
-  // completions of raw slot s's barrier per item
-  auto phases = [nz](int s) { return (nz + 4 + RAW - 1 - s) / RAW; };
+  const int nitem = Z_CUT ? A.cut.items() : A.nblk;
+  // completions of raw slot s's barrier by an item of n planes
+  auto phases = [](int n, int s) { return (n + 4 + RAW - 1 - s) / RAW; };
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
   R* sRaw = reinterpret_cast<R*>(smem_raw + S::raw);
@@ -431,11 +460,14 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
     for (int i = 0; i < RAW; ++i) mbar_init(bar + i, 1);
     fence_mbar_init();
   }
+  int wb = blockIdx.x, k0 = 0, nz = NB;   // this CTA's item: block, first plane, planes
+  if constexpr (Z_CUT) A.cut.item(blockIdx.x, wb, k0, nz);
   chain_wait();
   __syncthreads();
   int st = 0;
   // Persistent loop: this CTA starts with item blockIdx.x and then takes the next free item
-  // from the launch's counter; every item completes phases(s) phases of raw slot s's barrier.
+  // from the launch's counter; an item of nz planes completes phases(nz, s) phases of raw slot
+  // s's barrier.
   __shared__ int s_next;
   __shared__ int s_src[6], s_slot[6];   // face sources / register slots of the current block
   __shared__ R s_kc[12];                // per-(solve, level) constants, formed by thread 0
@@ -462,8 +494,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   const R kap0 = R(A.htc_kappa0);
   const R reta = R(A.eta);
   if (t == 0 && (int)blockIdx.x < nitem) {
-    const int i0 = (int)blockIdx.x >> zs;
-    const int b0 = A.wl ? A.wl[i0] : i0;
+    const int b0 = A.wl ? A.wl[wb] : wb;
 #pragma unroll
     for (int f = 0; f < 6; ++f) {
       s_src[f] = A.bd[b0].src[f];
@@ -474,10 +505,11 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   const int* src = s_src;
   const int* slot = s_slot;
   // work item w lies in pool block b (the work list of a batch skips the blocks of detached
-  // solves); the items of a block are consecutive
-  for (int w = blockIdx.x, jb = 0; w < nitem; ++jb) {
-  const int b = A.wl ? A.wl[w >> zs] : w >> zs;
-  const int k0 = (w & ((1 << zs) - 1)) * nz, k1 = k0 + nz;
+  // solves)
+  unsigned odd = 0;   // bit s: raw slot s's barrier has completed an odd number of phases before this item
+  for (int w = blockIdx.x; w < nitem;) {
+  const int b = A.wl ? A.wl[wb] : wb;
+  const int k1 = k0 + nz;
   const int sv = A.solve_of ? A.solve_of[b] : 0;
   const BlockDesc& bd = A.bd[b];
   // a block whose faces are corrected after this launch gets its CFL maxima and the second GLM
@@ -548,7 +580,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
     const int q = p - k0 + 2;
     R u[NT];
     if (plane_tma(p)) {
-      if (!mbar_wait(bar + (q % RAW), ((q / RAW) + jb * phases(q % RAW)) & 1, WAIT_LIMIT)) st |= ST_ETIMEOUT;
+      if (!mbar_wait(bar + (q % RAW), ((q / RAW) + ((odd >> (q % RAW)) & 1)) & 1, WAIT_LIMIT)) st |= ST_ETIMEOUT;
       const R* r = sRaw + (size_t)(q % RAW) * NT * 256 + cell2;
 #pragma unroll
       for (int v = 0; v < NT; ++v) u[v] = r[v * 256];
@@ -682,7 +714,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   if (t == 0) {
     fence_proxy_async();
     for (int p = RAW - 2; p <= (RAW == 3 ? 2 : 3); ++p)
-      if (p <= nz + 1) issue(k0 + p);
+      if (k0 + p <= k1 + 1) issue(k0 + p);
   }
   convert_own(k0);
   R fzd[NV], fzu[NV], hz[NV];
@@ -704,8 +736,8 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   __syncthreads();   // plane k0 of the ring (interior and halo) is complete
   if (RAW == 3 && t == 0) {   // raw slots of planes k0 and k0 + 1, converted above
     fence_proxy_async();
-    if (3 <= nz + 1) issue(k0 + 3);
-    if (4 <= nz + 1) issue(k0 + 4);
+    if (k0 + 3 <= k1 + 1) issue(k0 + 3);
+    if (k0 + 4 <= k1 + 1) issue(k0 + 4);
   }
 
   R ssum = R(0), smax = R(0);
@@ -1025,7 +1057,9 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
     const int nx = A.work ? (int)gridDim.x + atomicAdd(A.work, 1) : w + (int)gridDim.x;
     s_next = nx;
     if (nx < nitem) {
-      const int bn = A.wl ? A.wl[nx >> zs] : nx >> zs;
+      int in = nx, k_, n_;
+      if constexpr (Z_CUT) A.cut.item(nx, in, k_, n_);
+      const int bn = A.wl ? A.wl[in] : in;
 #pragma unroll
       for (int f = 0; f < 6; ++f) {
         s_src[f] = A.bd[bn].src[f];
@@ -1035,6 +1069,11 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   }
   __syncthreads();       // ring, raw slots, flux buffers and reduction scratch are reused next
   w = s_next;
+  if (w >= nitem) break;
+#pragma unroll
+  for (int s = 0; s < RAW; ++s) odd ^= (unsigned)(phases(k1 - k0, s) & 1) << s;
+  wb = w;
+  if constexpr (Z_CUT) A.cut.item(w, wb, k0, nz);
   }
   if (st) atomicOr(A.status, st);
 }
