@@ -80,10 +80,11 @@ struct StageArgs {
   int layout = 0;               // staging layout (STAGE_LAYOUT_*), 0: the default for the physics
   double eta = 0.0;             // resistive mhd: uniform resistivity
   const int* wl = nullptr;      // work list: pool block of each of the nblk work items (nullptr: identity)
-  // FP32 copies of the equation parameters and the combine weights, formed on the host at
-  // launch (stage_go), so that the FP32 kernel never forms them from the FP64 fields (the
+  // The equation parameters in both precisions and FP32 copies of the combine weights, formed on
+  // the host at launch (stage_go), so that no kernel forms them from the fields above (the
   // compiler may recompute such values at every use instead of holding them in registers)
   PhysParamsT<float> ppf;
+  PhysParamsT<double> ppd;
   float fa = 0.0f, fb = 0.0f;
   int combine = 0;
   StageCut cut;                 // the launch's work items, set by stage_go
@@ -409,6 +410,13 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   // 0.96 ms per stage and a 128^3 MHD one from 5.5 to 4.6 ms. FP32 kernels are bound by
   // instruction issue and barriers, and form them twice.
   constexpr bool SHARED_SLOPES = sizeof(R) == 8;
+  // FP64: the face buffers hold the fluxes as they are, and the update takes dt / dx times their
+  // differences (formed once per solve and level) instead of scaling every face by 1 / dx and
+  // the sum by dt: 9 instead of 11 FP64 operations per variable and cell. With one root for the
+  // signal speed of a state (rsqrt_div), the z-differences carried and the parameters from the
+  // host: HD 210 blocks 826 -> 790 us a launch, MHD 512 blocks 4270 -> 4127, SRHD 512 blocks 3306
+  // -> 3252.
+  constexpr bool FLUX_DT = sizeof(R) == 8 && !P::SOURCE;
   // A work item is planes k0 .. k0 + nz - 1 of a block (without Z_CUT the whole block): it reads
   // planes k0 - 2 .. k0 + nz + 1, TMA sequence 0 .. nz + 3.
   const int nitem = Z_CUT ? A.cut.items() : A.nblk;
@@ -481,7 +489,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
     ra = A.fa;
     rb = A.fb;
   } else {
-    pp.set(A.gamma, 0.0);
+    pp = A.ppd;
     ra = R(A.a);
     rb = R(A.b);
   }
@@ -490,6 +498,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   constexpr uint32_t PLANE_BYTES = (uint32_t)(sizeof(R) * NT * 256);
   int key_sv = -1, key_lev = -1;
   R idx = R(0), idy = R(0), idz = R(0), rdt = R(0), glm_fr = R(1);
+  R wx = R(0), wy = R(0), wz = R(0);   // FLUX_DT: dt (flux unit) / dx along x, y, z
   R rq4 = R(0);                        // 1 / tau = 1 / (4 dt) of the conduction relaxation
   const R kap0 = R(A.htc_kappa0);
   const R reta = R(A.eta);
@@ -543,6 +552,11 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
     idy = s_kc[1];
     idz = s_kc[2];
     rdt = s_kc[3];
+    if constexpr (FLUX_DT) {
+      wx = FU * rdt * idx;
+      wy = FU * rdt * idy;
+      wz = FU * rdt * idz;
+    }
     rq4 = s_kc[4];
     glm_fr = s_kc[8];
     pp.ch = s_kc[9];
@@ -658,6 +672,10 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
       for (int v = 0; v < NV; ++v) d[v * 400] = pr[v];
     }
   };
+  // FP64 with one CTA per SM (registers to spare): the difference of planes k + 1 and k + 2 is
+  // carried to the next plane too (MHD 512 blocks 4174 -> 4127 us)
+  constexpr bool CARRY_Z = sizeof(R) == 8 && MINB == 1;
+  R dz[CARRY_Z ? NV : 1];
   // z-face flux at k + 1/2 of this column. hz holds half the limited slope of plane k
   // (from the previous z-face, where plane k was the upper cell) and leaves with that of
   // plane k + 1, so each plane's z-slope is formed once.
@@ -669,7 +687,9 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       bq[v] = r1[v * 400]; c[v] = r2[v * 400]; d[v] = r3[v * 400];
-      const R h = v < P::NREC ? half_slope<R, LIM>(c[v] - bq[v], d[v] - c[v]) : R(0);
+      const R up = d[v] - c[v];
+      const R h = v < P::NREC ? half_slope<R, LIM>(CARRY_Z ? dz[CARRY_Z ? v : 0] : c[v] - bq[v], up) : R(0);
+      if constexpr (CARRY_Z) dz[v] = up;
       pl[v] = bq[v] + hz[v];
       pr[v] = c[v] - h;
       hz[v] = h;
@@ -723,8 +743,11 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
     const R* r1 = ring(k0 - 1) + cellp;
     const R* r2 = ring(k0) + cellp;
 #pragma unroll
-    for (int v = 0; v < NV; ++v)
-      hz[v] = v < P::NREC ? half_slope<R, LIM>(r1[v * 400] - r0[v * 400], r2[v * 400] - r1[v * 400]) : R(0);
+    for (int v = 0; v < NV; ++v) {
+      const R up = r2[v * 400] - r1[v * 400];
+      hz[v] = v < P::NREC ? half_slope<R, LIM>(r1[v * 400] - r0[v * 400], up) : R(0);
+      if constexpr (CARRY_Z) dz[v] = up;
+    }
   }
   convert_own(k0 + 1);
   zface(k0 - 1, fzd, hz);
@@ -897,7 +920,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
         riemann<P, R, 0, FLUX>(pl, pr, f, pp);
         if constexpr (SHARED_SLOPES) __syncthreads();   // every x-slope has been read
 #pragma unroll
-        for (int v = 0; v < NV; ++v) sFx[v * FXN + fx0] = f[v] * (FU * idx);
+        for (int v = 0; v < NV; ++v) sFx[v * FXN + fx0] = FLUX_DT ? f[v] : f[v] * (FU * idx);
         if (FR && tx == 0 && slot[0] >= 0) {
 #pragma unroll
           for (int v = 0; v < NV; ++v) FR[((size_t)slot[0] * NV + v) * 256 + k * 16 + ty] = FU * f[v];
@@ -906,7 +929,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
         riemann<P, R, 1, FLUX>(pl, pr, f, pp);
         if constexpr (SHARED_SLOPES) __syncthreads();   // every y-slope has been read
 #pragma unroll
-        for (int v = 0; v < NV; ++v) sFy[v * FYN + fy0] = f[v] * (FU * idy);
+        for (int v = 0; v < NV; ++v) sFy[v * FYN + fy0] = FLUX_DT ? f[v] : f[v] * (FU * idy);
         if (FR && ty == 0 && slot[2] >= 0) {
 #pragma unroll
           for (int v = 0; v < NV; ++v) FR[((size_t)slot[2] * NV + v) * 256 + k * 16 + tx] = FU * f[v];
@@ -955,7 +978,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
         swap_xy<P, R>(f, yd);
         const R ids = FU * (yd ? idy : idx);
 #pragma unroll
-        for (int v = 0; v < NV; ++v) dstp[v * ns] = f[v] * ids;
+        for (int v = 0; v < NV; ++v) dstp[v * ns] = FLUX_DT ? f[v] : f[v] * ids;
         const int sl = slot[1 + 2 * fs];
         if (FR && sl >= 0) {
 #pragma unroll
@@ -1015,13 +1038,23 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
         for (int v = 0; v < NV; ++v) {
           const R lx = sFx[v * FXN + fx1] - sFx[v * FXN + fx0];
           const R ly = sFy[v * FYN + fy1] - sFy[v * FYN + fy0];
-          const R lz = (fzu[v] - fzd[v]) * (FUZ * idz);
-          R L = -((lx + ly) + lz);
-          if constexpr (RESP) {
-            if (v >= P::BOFF && v < P::BOFF + 3) L = L + rsrc[v - P::BOFF];
-            if (v == P::IE) L = L + rsrc[3];
+          R val = US_GLOBAL ? usk[US_GLOBAL ? v : 0] : raw[v * 256];
+          if constexpr (FLUX_DT) {
+            R d = wx * lx + wy * ly + wz * (fzu[v] - fzd[v]);
+            if constexpr (RESP) {
+              if (v >= P::BOFF && v < P::BOFF + 3) d = d - rdt * rsrc[v - P::BOFF];
+              if (v == P::IE) d = d - rdt * rsrc[3];
+            }
+            val = val - d;
+          } else {
+            const R lz = (fzu[v] - fzd[v]) * (FUZ * idz);
+            R L = -((lx + ly) + lz);
+            if constexpr (RESP) {
+              if (v >= P::BOFF && v < P::BOFF + 3) L = L + rsrc[v - P::BOFF];
+              if (v == P::IE) L = L + rsrc[3];
+            }
+            val = val + rdt * L;
           }
-          R val = (US_GLOBAL ? usk[US_GLOBAL ? v : 0] : raw[v * 256]) + rdt * L;
           if (combine) val = ra * unk[v] + rb * val;
           out[v] = val;
           fzd[v] = fzu[v];

@@ -158,6 +158,7 @@ static cudaError_t stage_go_layout(const StageArgs& a, cudaStream_t s) {
   int grid = a.grid > 0 ? a.grid : MINB * sms;
   if (grid > args.cut.items()) grid = args.cut.items();
   args.ppf.set(a.gamma, 0.0);
+  args.ppd.set(a.gamma, 0.0);
   args.fa = (float)a.a;
   args.fb = (float)a.b;
   args.combine = a.a != 0.0 ? 1 : 0;
