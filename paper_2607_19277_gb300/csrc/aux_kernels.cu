@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(256) fixup_kernel(R* __restrict__ U, const R* 
 // with corrected faces, where one CTA per block spent 16 us on 16 cells in sequence.
 constexpr int SPEED_PARTS = 4;
 template <template <typename> class PT, typename R>
-__global__ void __launch_bounds__(256) speeds_kernel(const R* __restrict__ U,
+__global__ void __launch_bounds__(256) speeds_kernel(const R* U,
                                                       const BlockDesc* __restrict__ bd,
                                                       const PhysParamsT<R> pp,   // formed on the host
                                                       unsigned long long* speeds, int* status,
@@ -280,8 +280,8 @@ __global__ void set_dt_kernel(unsigned long long* speeds, double* dtch, double d
 // One CTA per block: thread 0 forms the factor in FP64, the CTA scales psi in the stencil
 // precision with 16-byte accesses (psi of a block is 4096 contiguous values).
 template <typename R>
-__global__ void __launch_bounds__(256) glm_decay_kernel(R* __restrict__ U, const BlockDesc* __restrict__ bd,
-                                                         const double* __restrict__ dtch, double alpha,
+__global__ void __launch_bounds__(256) glm_decay_kernel(R* U, const BlockDesc* __restrict__ bd,
+                                                         const double* dtch, double alpha,
                                                          const int* __restrict__ solve_of,
                                                          const int* __restrict__ wl) {
   __shared__ R s_f;
@@ -585,8 +585,7 @@ __global__ void __launch_bounds__(256, 4) regrid_kernel(const R* __restrict__ Uo
 // cells per solve from these primitives, as the stage kernel's fused reduction would have
 // from the same state at the end of the previous step.
 template <template <typename> class PT, typename R>
-__global__ void __launch_bounds__(256) prim_pass_kernel(const R* __restrict__ U, R* __restrict__ W,
-                                                        const R* __restrict__ G, R* __restrict__ WG,
+__global__ void __launch_bounds__(256) prim_pass_kernel(const R* U, R* W, const R* G, R* WG,
                                                         const int* __restrict__ wl, int nwork,
                                                         PhysParamsT<R> pp, int* status,
                                                         const BlockDesc* __restrict__ bd,

@@ -145,9 +145,9 @@ __device__ __forceinline__ R cool_temperature(R rho, R T, R dt, const CoolDev& c
 // conversion shared the same way).
 constexpr int COOL_PARTS = 4;
 template <template <typename> class PT, typename R>
-__global__ void __launch_bounds__(256) cooling_kernel(R* __restrict__ U, const BlockDesc* __restrict__ bd,
+__global__ void __launch_bounds__(256) cooling_kernel(R* U, const BlockDesc* __restrict__ bd,
                                                        CoolDev c, const R* __restrict__ seg,
-                                                       const double* __restrict__ dtch, double frac,
+                                                       const double* dtch, double frac,
                                                        const PhysParamsT<R> pp,   // formed on the host
                                                        unsigned long long* speeds,
                                                        int* status, const int* __restrict__ solve_of) {

@@ -94,7 +94,7 @@ struct StageArgs {
 // Conserved + auxiliary values of the cell (x, y, z) of block b in the halo view: the
 // interior, a same-level neighbour's interior, a physical boundary image or a ghost slot.
 template <class P, typename R>
-__device__ __forceinline__ void load_cell(const R* __restrict__ U, const R* __restrict__ G,
+__device__ __forceinline__ void load_cell(const R* U, const R* G,
                                           const int* src, int b, int x, int y, int z, R* u) {
   constexpr int NT = P::NV + P::NA;
   int f = -1;
@@ -140,7 +140,11 @@ __device__ __forceinline__ void load_cell(const R* __restrict__ U, const R* __re
 
 // Chained launches (launch_chained): wait until the kernel before this one on the stream has
 // completed and its writes are visible (nothing to wait for in a plain launch), then let the
-// next one take its place.
+// next one take its place. The kernel's lifetime begins before the wait, while the one before still
+// writes, so what any kernel of a step writes (states, ghost slots, primitives, dt, maxima) is read
+// with ordinary loads here: the read-only path (__ldg, or const __restrict__, which also lets the
+// compiler move a load across the wait) is for memory that nothing writes during the kernel's
+// lifetime, i.e. the tables that only copies write (bd, wl, solve_of, seg).
 __device__ __forceinline__ void chain_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -268,7 +272,7 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // stride there (same pointer rules as load_cell); *neg_d is the dimension whose normal
 // components a reflecting boundary negates, or -1.
 template <class P, typename R>
-__device__ __forceinline__ const R* cell_addr(const R* __restrict__ U, const R* __restrict__ G,
+__device__ __forceinline__ const R* cell_addr(const R* U, const R* G,
                                               const int* src, int b, int x, int y, int z, int* vstride,
                                               int* neg_d) {
   constexpr int NT = P::NV + P::NA;
@@ -429,14 +433,14 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   R* sFx0 = reinterpret_cast<R*>(smem_raw + S::fx);
   R* sFy0 = reinterpret_cast<R*>(smem_raw + S::fy);
 
-  const R* __restrict__ Us = static_cast<const R*>(A.Us);
-  const R* __restrict__ Un = static_cast<const R*>(A.Un);
-  R* __restrict__ Uo = static_cast<R*>(A.Uout);
-  const R* __restrict__ G = static_cast<const R*>(A.gs);
-  R* __restrict__ FR = static_cast<R*>(A.fr);
+  const R* Us = static_cast<const R*>(A.Us);
+  const R* Un = static_cast<const R*>(A.Un);
+  R* Uo = static_cast<R*>(A.Uout);
+  const R* G = static_cast<const R*>(A.gs);
+  R* FR = static_cast<R*>(A.fr);
   // what the ring is filled from: U_s and its ghost slots, or their primitives
-  const R* __restrict__ Rs = PRIMIN ? static_cast<const R*>(A.W) : Us;
-  const R* __restrict__ Rg = PRIMIN ? static_cast<const R*>(A.WG) : G;
+  const R* Rs = PRIMIN ? static_cast<const R*>(A.W) : Us;
+  const R* Rg = PRIMIN ? static_cast<const R*>(A.WG) : G;
 
   const int t = threadIdx.x;
   const int warp = t >> 5;
@@ -837,21 +841,23 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
       for (int i = 0; i < 3; ++i) rsrc[i] = reta * lap[i];
       rsrc[3] = reta * (jj + blap);
     }
-    // U^n of cell (tx, ty, k) for the stage combine, loaded now so that the face work of
-    // this phase covers its latency
-    // likewise U_s of the cell where no raw plane holds it then (read at the update it held up
-    // every plane: SRHD 332 -> 317 us a launch of 1584 FP32 blocks)
+    // U_s of cell (tx, ty, k) where no raw plane holds it at the update, from L2 (where the TMA
+    // has passed it through; ordinary and L2 loads of U_s and U^n in any combination were within
+    // 1% of each other on a 256^3 MHD request, 63.5 to 64.4 ms; the read-only path, which a
+    // chained kernel may not use, 63.1), and U^n for the stage combine: loaded now, so that the
+    // face work of this phase covers their latency (U_s read at the update itself held up every
+    // plane: SRHD 332 us a launch of 1584 FP32 blocks, not 317)
     R usk[US_GLOBAL ? NV : 1];
     if constexpr (US_GLOBAL) {
       const R* ps = Us + (size_t)b * NT * NCELL + (size_t)k * 256 + cell2;
 #pragma unroll
-      for (int v = 0; v < NV; ++v) usk[v] = __ldg(ps + (size_t)v * NCELL);
+      for (int v = 0; v < NV; ++v) usk[v] = __ldcg(ps + (size_t)v * NCELL);
     }
     R unk[NV];
     if (combine) {
       const R* pn = Un + (size_t)b * NT * NCELL + (size_t)k * 256 + cell2;
 #pragma unroll
-      for (int v = 0; v < NV; ++v) unk[v] = __ldg(pn + (size_t)v * NCELL);
+      for (int v = 0; v < NV; ++v) unk[v] = pn[(size_t)v * NCELL];
     }
     {
       R f[NV];
