@@ -277,7 +277,9 @@ struct MhdPhys {
   // Conserved state, flux along D (without those of B_d and psi, which riemann sets from the
   // face values) and the interval of the speeds of a face state. FP64: the fast speed from
   // S = gamma p + B^2, cf^2 = (S + sqrt(S^2 - 4 gamma p B_d^2)) / (2 rho), which divides by the
-  // density once; FP32 keeps every square near a^4, whose range it can hold.
+  // density once, for S from 2^-480 (S^2 keeps its bits below its terms down to there) to below
+  // 2^511 (S^2 does not overflow; the subtrahend is at most S^2); elsewhere, and in FP32, from
+  // quantities divided by the density (waves), whose squares are near a^4.
   template <int D>
   __device__ static __forceinline__ void side(const R* p, R* u, R* f, R& mid, R& half, const PhysParamsT<R>& pp) {
     const R vd = p[1 + D], bd = p[5 + D];
@@ -305,8 +307,13 @@ struct MhdPhys {
     f[5 + D] = R(0);
     f[8] = R(0);
     if constexpr (sizeof(R) == 8) {
+      constexpr unsigned LO = (1023u - 480u) << 20, HI = (1023u + 511u) << 20;   // high words
       const R gp = pp.gamma * p[4];
       const R s = gp + b2;
+      if ((unsigned)__double2hiint(s) - LO >= HI - LO) {   // a negative or non-finite S as well
+        waves<D>(p, mid, half, pp);
+        return;
+      }
       const R disc = rmax(s * s - (R(4) * gp) * (bd * bd), R(0));
       mid = vd;
       half = rsqrt_div(R(0.5) * (s + rsqrt_(disc)), p[0]);

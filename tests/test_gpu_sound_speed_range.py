@@ -1,8 +1,11 @@
-"""The FP64 hydro speed sqrt(gamma p / rho) takes the root of the product p rho where that is a
-normal number and the quotient's root elsewhere: a state scaled by a power of two (density,
-momentum and energy; the equations are homogeneous in it) that takes p rho out of that range
-gives the scaled results. Each of the two roots is within 2 ulp, and the stencil damps a speed's error to its
-share of the flux, so two steps stay within 1e-14 of one another."""
+"""The FP64 signal speeds are formed from products that have the square of the state's scale: the
+hydro speed sqrt(gamma p / rho) from the root of p rho where that is a normal number and from the
+quotient's root elsewhere, the MHD face's fast speed from S = gamma p + B^2 where S^2 keeps its
+bits and from quantities divided by the density elsewhere. The equations are homogeneous: a state
+scaled by a power of two (density, momentum and energy by s, B and psi by sqrt(s)) gives the scaled
+results, also where it takes those products out of the range. Each of the roots is within 2 ulp,
+and the stencil damps a speed's error to its share of the flux, so two steps stay within 1e-14 of
+one another."""
 import numpy as np
 import pytest
 
@@ -11,17 +14,13 @@ from paper_2607_19277_gb300 import agile, workloads as W
 pytestmark = pytest.mark.gpu
 
 
-def _steps(scale, flux):
-    m = agile.Mesh(agile.make_config(physics="hd", limiter="minmod", flux=flux, rk=2, real_bytes=8,
+def _steps(physics, exponent, flux):
+    nv = agile.NVAR[agile.PHYSICS[physics]]
+    by = np.ldexp(1.0, np.where(np.arange(nv) >= 5, exponent // 2, np.where(np.arange(nv) % 4, 0, exponent)))
+    m = agile.Mesh(agile.make_config(physics=physics, limiter="minmod", flux=flux, rk=2, real_bytes=8,
                                      base_blocks=(2, 2, 2)))
-    ic = W.random_smooth(5, 11, "hd")
-
-    def scaled(x, y, z):
-        p = np.array(ic(x, y, z))
-        p[[0, 4]] *= scale
-        return p
-
-    m.set_state(scaled)
+    ic = W.random_smooth(nv, 11, physics)
+    m.set_state(lambda x, y, z: (np.array(ic(x, y, z)).T * by).T)   # rho, p by s; B, psi by sqrt(s)
     for _ in range(2):
         m.step()
     cons = m.get_state()[2]
@@ -30,10 +29,13 @@ def _steps(scale, flux):
 
 
 @pytest.mark.parametrize("flux", ["tvdlf", "hll"])
-@pytest.mark.parametrize("exponent", [-600, -511, 500, 600])
-def test_scaled_state(flux, exponent):
-    one = _steps(1.0, flux)
-    got = _steps(2.0 ** exponent, flux) * 2.0 ** -exponent
-    for v in range(5):
-        err = np.abs(got[:, v] - one[:, v]).sum() / max(np.abs(one[:, v]).sum(), np.abs(one[:, 0]).sum())
+@pytest.mark.parametrize("physics,exponent", [("hd", -600), ("hd", -511), ("hd", 500), ("hd", 600),
+                                              ("mhd", -600), ("mhd", -510), ("mhd", -400), ("mhd", 500), ("mhd", 600)])
+def test_scaled_state(physics, flux, exponent):
+    one = _steps(physics, 0, flux)
+    got = _steps(physics, exponent, flux)
+    for v in range(one.shape[1]):
+        back = np.ldexp(got[:, v], -(exponent // 2 if v >= 5 else exponent))
+        own = np.abs(one[:, v]).sum()
+        err = np.abs(back - one[:, v]).sum() / max(own, np.abs(one[:, 5 if v >= 5 else 0]).sum())
         assert err < 1e-14, (v, err)
