@@ -450,6 +450,22 @@ agile_status agile_selftest_bounded_wait(void* stream, unsigned int limit, int* 
 agile_status agile_selftest_rcp64(const double* s, const double* a, size_t n, void* stream, double* max_ulps,
                                   double* max_rel);
 
+/* The FP64 stencil's own roots and comparisons, evaluated on the device for the n elements of the
+ * HOST arrays a and b into the host array out (1 <= n <= 2^26; b is read by every op, used by
+ * those of two arguments; any value may be passed). Synchronises `stream` (a cudaStream_t, NULL
+ * for the default stream). AGILE_EINVAL for a null array, an n or an op out of range. */
+enum {
+  AGILE_FP64_SQRT = 0,           /* sqrt(a): within 0.52 ulp */
+  AGILE_FP64_SQRT_QUOTIENT = 1,  /* sqrt(a / b), positive a and b, |b| normal and below 2^1022:
+                                  * within 1.02 ulp where a b is a normal number and a >= 2^-959,
+                                  * else within 1.55 ulp where a / b is a normal number */
+  AGILE_FP64_MIN = 2,            /* the smaller; of a NaN and a number the number; -0 below +0 */
+  AGILE_FP64_MAX = 3,
+  AGILE_FP64_POSITIVE = 4,       /* 1 where a > 0, else 0 */
+  AGILE_FP64_NOT_NONNEGATIVE = 5 /* 1 unless a >= 0 (a NaN gives 1), else 0 */
+};
+agile_status agile_selftest_fp64(int op, const double* a, const double* b, size_t n, void* stream, double* out);
+
 /* Message of the last failed call on this mesh (static storage owned by the mesh). */
 const char* agile_last_error(const agile_mesh* mesh);
 

@@ -35,7 +35,7 @@ EXPORTS = ["agile_mesh_create", "agile_mesh_destroy", "agile_set_state", "agile_
            "agile_conserved_sums_noalloc", "agile_set_cooling", "agile_estimate",
            "agile_get_halo", "agile_sync", "agile_set_kernel_timing", "agile_kernel_timing",
            "agile_phase_timing",
-           "agile_selftest_bounded_wait", "agile_selftest_rcp64", "agile_last_error", "agile_version",
+           "agile_selftest_bounded_wait", "agile_selftest_rcp64", "agile_selftest_fp64", "agile_last_error", "agile_version",
            "agile_batch_create", "agile_batch_destroy", "agile_batch_layout",
            "agile_batch_set_state", "agile_batch_step", "agile_batch_cfl_dt", "agile_batch_copy_solve",
            "agile_batch_autotune", "agile_batch_regrid", "agile_batch_regrid_flags",
@@ -111,6 +111,7 @@ def load(path: str = LIB_PATH):
         "agile_phase_timing": (C.c_int, [P, dp, C.POINTER(C.c_longlong)]),
         "agile_selftest_bounded_wait": (C.c_int, [P, C.c_uint, ip]),
         "agile_selftest_rcp64": (C.c_int, [dp, dp, C.c_size_t, P, dp, dp]),
+        "agile_selftest_fp64": (C.c_int, [C.c_int, dp, dp, C.c_size_t, P, dp]),
         "agile_last_error": (C.c_char_p, [P]),
         "agile_version": (C.c_char_p, []),
         "agile_batch_create": (C.c_int, [C.POINTER(agile_config), C.c_int, C.POINTER(agile_allocator), P, C.POINTER(P)]),
@@ -216,6 +217,22 @@ def check_rcp64(s, a):
     st = lib.agile_selftest_rcp64(_dptr(s), _dptr(a), s.size, None, C.byref(mu), C.byref(mr))
     _check(lib, None, st)
     return mu.value, mr.value
+
+
+FP64_OPS = {"sqrt": 0, "sqrt_quotient": 1, "min": 2, "max": 3, "positive": 4, "not_nonnegative": 5}
+
+
+def eval_fp64(op, a, b=None):
+    """The FP64 stencil's own root or comparison (a key of FP64_OPS) of the elements of a (and b),
+    formed on the device (agile_selftest_fp64)."""
+    lib = load()
+    a = np.ascontiguousarray(a, dtype=np.float64).ravel()
+    b = a if b is None else np.ascontiguousarray(b, dtype=np.float64).ravel()
+    if a.shape != b.shape:
+        raise ValueError("a and b differ in size")
+    out = np.empty_like(a)
+    _check(lib, None, lib.agile_selftest_fp64(FP64_OPS[op], _dptr(a), _dptr(b), a.size, None, _dptr(out)))
+    return out
 
 
 def _check(lib, mesh_ptr, st):
