@@ -47,7 +47,7 @@ struct agile_mesh {
   unsigned long long* d_speeds = nullptr;
   double* d_dtch = nullptr;
   int* d_work = nullptr;            // per-stage item counters of the persistent launches
-  StageCut cut;                     // work items of the stage launches (stage_go)
+  StageCutCache cut;                // work items of the stage launches (stage_go)
   int* d_vars = nullptr;
   double* d_weights = nullptr;
   bool speeds_valid = false;
@@ -1190,7 +1190,7 @@ struct agile_batch {
   int grid = 0;                     // persistent CTAs of the stage launches (0: default)
   bool dynamic = true;              // blocks taken from an atomic counter (else strided)
   int layout = 0;                   // staging layout of the stage kernel (0: the default)
-  StageCut cut;                     // work items of the stage launches (stage_go)
+  StageCutCache cut;                // work items of the stage launches (stage_go)
   // refinement: ghost slots, flux registers and their tasks of all solves (indices offset)
   void* G = nullptr;
   void* FR = nullptr;

@@ -16,40 +16,11 @@
 #include "agile_internal.h"
 #include "pair.cuh"
 #include "physics.cuh"
+#include "stage_cut.h"
 
 namespace agile {
 
 enum : int { STAGE_LAYOUT_RING4 = 1, STAGE_LAYOUT_RING5_DB = 2, STAGE_LAYOUT_RING3_DB = 3 };
-
-// Work items of a launch over nblk blocks: the first n1 blocks whole, of the others m items of a
-// planes each, then (behind all of those) one of the 16 - m a planes left, if any. Sizes fall
-// along the list, so that CTAs taking the next free item end close together.
-struct StageCut {
-  int nblk = -1;
-  int n1 = 0, a = NB, m = 1;
-  unsigned long long inv_m = 1ull << 32;   // ceil(2^32 / m): exact for items below 2^28
-  __host__ __device__ int rest() const { return NB - m * a; }
-  __host__ __device__ int items() const { return n1 + (nblk - n1) * (rest() > 0 ? m + 1 : m); }
-  __host__ __device__ bool whole() const { return n1 == nblk || a == NB; }
-  // block (index into the work list), first plane and planes of item w
-  __host__ __device__ void item(int w, int& blk, int& k0, int& nz) const {
-    const int nr = nblk - n1;
-    if (w < n1) {
-      blk = w;
-      k0 = 0;
-      nz = NB;
-    } else if (w - n1 < nr * m) {
-      const int v = w - n1, q = (int)((unsigned long long)(unsigned)v * inv_m >> 32);   // v / m
-      blk = n1 + q;
-      k0 = (v - q * m) * a;
-      nz = a;
-    } else {
-      blk = n1 + (w - n1 - nr * m);
-      k0 = m * a;
-      nz = rest();
-    }
-  }
-};
 
 struct StageArgs {
   const void* Us;           // stage input state (with aux)
@@ -88,7 +59,7 @@ struct StageArgs {
   float fa = 0.0f, fb = 0.0f;
   int combine = 0;
   StageCut cut;                 // the launch's work items, set by stage_go
-  StageCut* cut_cache = nullptr;  // host: the caller's copy, formed again when nblk changes
+  StageCutCache* cut_cache = nullptr;  // host: the caller's copy (required)
 };
 
 // Conserved + auxiliary values of the cell (x, y, z) of block b in the halo view: the
