@@ -466,6 +466,14 @@ enum {
 };
 agile_status agile_selftest_fp64(int op, const double* a, const double* b, size_t n, void* stream, double* out);
 
+/* The relativistic primitive recovery of the FP32 stencil, evaluated on the device for the n cells of
+ * the HOST arrays cons[n][5] (D, m, tau) and start[n] (the stored xi the iteration begins at, any
+ * value) into out[n][8]: rho, u (3), p, xi, Gamma and 1 where the last step ran in pairs of FP32
+ * numbers, 0 where in FP64, -1 where the recovery failed or is unphysical. 1 <= n <= 2^26, gamma > 1,
+ * eos AGILE_EOS_*, else AGILE_EINVAL. Synchronises `stream`. */
+agile_status agile_selftest_recover32(int eos, double gamma, const float* cons, const float* start, size_t n,
+                                      void* stream, float* out);
+
 /* Message of the last failed call on this mesh (static storage owned by the mesh). */
 const char* agile_last_error(const agile_mesh* mesh);
 

@@ -35,7 +35,8 @@ EXPORTS = ["agile_mesh_create", "agile_mesh_destroy", "agile_set_state", "agile_
            "agile_conserved_sums_noalloc", "agile_set_cooling", "agile_estimate",
            "agile_get_halo", "agile_sync", "agile_set_kernel_timing", "agile_kernel_timing",
            "agile_phase_timing",
-           "agile_selftest_bounded_wait", "agile_selftest_rcp64", "agile_selftest_fp64", "agile_last_error", "agile_version",
+           "agile_selftest_bounded_wait", "agile_selftest_rcp64", "agile_selftest_fp64",
+           "agile_selftest_recover32", "agile_last_error", "agile_version",
            "agile_batch_create", "agile_batch_destroy", "agile_batch_layout",
            "agile_batch_set_state", "agile_batch_step", "agile_batch_cfl_dt", "agile_batch_copy_solve",
            "agile_batch_autotune", "agile_batch_regrid", "agile_batch_regrid_flags",
@@ -112,6 +113,8 @@ def load(path: str = LIB_PATH):
         "agile_selftest_bounded_wait": (C.c_int, [P, C.c_uint, ip]),
         "agile_selftest_rcp64": (C.c_int, [dp, dp, C.c_size_t, P, dp, dp]),
         "agile_selftest_fp64": (C.c_int, [C.c_int, dp, dp, C.c_size_t, P, dp]),
+        "agile_selftest_recover32": (C.c_int, [C.c_int, C.c_double, C.POINTER(C.c_float), C.POINTER(C.c_float),
+                                             C.c_size_t, P, C.POINTER(C.c_float)]),
         "agile_last_error": (C.c_char_p, [P]),
         "agile_version": (C.c_char_p, []),
         "agile_batch_create": (C.c_int, [C.POINTER(agile_config), C.c_int, C.POINTER(agile_allocator), P, C.POINTER(P)]),
@@ -232,6 +235,22 @@ def eval_fp64(op, a, b=None):
         raise ValueError("a and b differ in size")
     out = np.empty_like(a)
     _check(lib, None, lib.agile_selftest_fp64(FP64_OPS[op], _dptr(a), _dptr(b), a.size, None, _dptr(out)))
+    return out
+
+
+def recover32(cons, start, gamma, eos="ideal"):
+    """Primitives (rho, u, p), xi, Gamma and the branch taken (1 pairs, 0 FP64, -1 failed) that the FP32
+    stencil's relativistic recovery gives for the conserved values cons[n][5] from the stored xi
+    start[n] (agile_selftest_recover32)."""
+    lib = load()
+    cons = np.ascontiguousarray(cons, dtype=np.float32).reshape(-1, 5)
+    start = np.ascontiguousarray(start, dtype=np.float32).ravel()
+    if len(cons) != len(start):
+        raise ValueError("cons and start differ in size")
+    out = np.empty((len(cons), 8), dtype=np.float32)
+    fp = C.POINTER(C.c_float)
+    _check(lib, None, lib.agile_selftest_recover32(EOS[eos], gamma, cons.ctypes.data_as(fp), start.ctypes.data_as(fp),
+                                                   len(cons), None, out.ctypes.data_as(fp)))
     return out
 
 

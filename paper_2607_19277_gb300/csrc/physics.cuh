@@ -473,6 +473,16 @@ struct SrhdPhysE {
   static constexpr bool GLM = false;
   using Eos = SrhdEos<R, EOS>;
 
+  // FP32 start x of the iteration from the stored xi, in the bracket [E, k E] formed in FP32 from the
+  // FP32 inputs, and their m^2.
+  __device__ static __forceinline__ void bracket(const float* u, float xi, const PhysParamsT<float>& pp, float& x,
+                                                 float& lo, float& hi, float& s2) {
+    lo = u[4] + u[0];
+    hi = (EOS == EOS_SYNGE ? 4.0f / 3.0f : pp.gamma) * lo;
+    x = xi > lo && xi < hi ? xi : 0.5f * (lo + hi);
+    s2 = u[1] * u[1] + u[2] * u[2] + u[3] * u[3];
+  }
+
   // The same Newton iteration in FP32, to |dxi| <= 1e-6 xi (at most 12 steps): in the FP32
   // stencil it moves the starting point close to the root, so that one more step in higher
   // precision (finish_pairs, or the FP64 iteration) reaches it.
@@ -517,15 +527,18 @@ struct SrhdPhysE {
   // the converged FP32 start x the step dx = -f(x) / f'(x), f evaluated in pairs from the FP32
   // inputs (which are exact), and the first-order update of every quantity by dx, the formulas
   // of the FP64 iteration below. GB300 runs FP64 at 1/64 of the FP32 rate, and these about 45
-  // FP64 operations are some 150 FP32 ones here. Pairs carry absolute errors of a few 2^-46 of
-  // xi (of 1 in v^2); the guards keep what the subtractions 1 - v^2 and xi / Gamma^2 - rho
-  // amplify below 2^-29 of the result, 1/32 of the FP32 rounding of the outputs: Gamma^2 <= 2^13
-  // and p >= 2^-14 xi, xi within 2^+-36 (no product's error is flushed to zero). Returns false,
-  // with nothing written, outside them or when the step is not below 1e-6 xi or leaves the
-  // bracket: the FP64 iteration takes the cell then. Against the root in extended precision
-  // (400,000 random states per range, Gamma to 60, p/rho from 1e-4 to 100, starts a few FP32
-  // roundings off) the largest and the rms errors of rho, u and p equal those of the FP64 step
-  // to three digits (rms 0.289 ulp at Gamma < 10). Recovery pass over 1466 blocks: 883 -> 96 us.
+  // FP64 operations are some 150 FP32 ones here. Pairs have 46 bits instead of 53: absolute errors
+  // of a few 2^-46 of xi (of 1 in v^2); the guards keep what the subtractions 1 - v^2 and
+  // xi / Gamma^2 - rho amplify of them below 2^-29 of the result, 1/32 of the FP32 rounding of the
+  // outputs: Gamma^2 <= 2^13 and p >= 2^-14 xi, xi within 2^+-36 (no product's error is flushed to
+  // zero). Returns false, with nothing written, outside them or when the step is not below 1e-6 xi
+  // or leaves the bracket: the FP64 iteration takes the cell then. The first-order update leaves
+  // out terms of some Gamma^4 (dxi / xi)^2, in FP64 and in pairs alike: at Gamma above 20 these, not
+  // the arithmetic, are the largest errors (up to 113 units of 2^-24 in Gamma on 400,000 states to
+  // Gamma = 88). Against the root in extended precision (400,000 random states per range, Gamma to
+  // 60, p/rho from 1e-4 to 100, starts a few FP32 roundings off) the largest and the rms errors of
+  // rho, u and p equal those of the FP64 step to three digits (rms 0.289 ulp at Gamma < 10).
+  // Recovery pass over 1466 blocks: 883 -> 96 us.
   __device__ static __forceinline__ bool finish_pairs(const float* u, float x, float lo, float hi, float* p,
                                                       float* aux, const PhysParamsT<float>& pp) {
     const float D = u[0];
@@ -593,12 +606,8 @@ struct SrhdPhysE {
                                                    int& st) {
     float xf = 0.0f;
     if constexpr (sizeof(R) == 4) {
-      // the FP32 start from the FP32 inputs in the bracket [E, k E] formed in FP32
-      const float ef = u[4] + u[0];
-      const float hif = (EOS == EOS_SYNGE ? 4.0f / 3.0f : (float)pp.gamma) * ef;
-      xf = aux[0];
-      if (!(xf > ef && xf < hif)) xf = 0.5f * (ef + hif);
-      const float s2f = u[1] * u[1] + u[2] * u[2] + u[3] * u[3];
+      float ef, hif, s2f;
+      bracket(u, aux[0], pp, xf, ef, hif, s2f);
       if (seed_f32(xf, u[0], s2f, ef, ef, hif, pp) && finish_pairs(u, xf, ef, hif, p, aux, pp)) return;
     }
     const double g = pp.gamma_d;

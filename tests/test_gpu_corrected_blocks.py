@@ -1,11 +1,13 @@
 """Blocks whose faces take the coarse-fine flux correction get their CFL maxima (and, for MHD, the
 second GLM half) in passes over them alone, every other block in the last stage's stores: the
 CFL step after a step on a three-level mesh equals the one reduced afresh from the same state,
-also where the fastest cell lies in such a block, on an edge of two corrected faces."""
+also where the fastest cell lies in such a block, on an edge of two corrected faces; and psi, which
+the second half multiplies, agrees with the oracle's in the corrected blocks as in the others."""
 import numpy as np
 import pytest
 
 from paper_2607_19277_gb300 import agile, workloads as W
+from parity_util import TOL_FP32, TOL_FP64, force_refine, gpu_mesh, oracle_solver
 
 pytestmark = pytest.mark.gpu
 
@@ -45,3 +47,32 @@ def test_cfl_after_a_step(physics, rb, hot):
     # the same maxima of the same cells; the two kernels may contract products differently
     ulp = 2.0 ** -52 if rb == 8 else 2.0 ** -22
     assert a == pytest.approx(b, rel=4 * ulp)
+
+
+@pytest.mark.parametrize("rb,tol", [(8, TOL_FP64), (4, TOL_FP32)])
+def test_second_glm_half(rb, tol):
+    spec = dict(physics="mhd", limiter="minmod", flux="hll", rk=2, base_blocks=(3, 2, 2), bc=("outflow",) * 6,
+                max_level=3)
+    ic = W.random_smooth(9, 9, "mhd")
+    o, m = oracle_solver(spec), gpu_mesh(spec, rb)
+    o.set_state(ic)
+    m.set_state(ic)
+    force_refine(o, m, {(1, 1, 0, 0), (1, 0, 1, 0)})
+    force_refine(o, m, {(2, 2, 1, 1)})
+    m.set_state_blocks(o.get_state()[2])
+    for _ in range(2):
+        dt = o.cfl_dt()
+        o.step(dt)
+        m.step(dt)
+    lev, ijk, g = m.get_state()
+    r = o.get_state()[2]
+    m.close()
+    keys = {(l, *c) for l, c in zip(lev.tolist(), ijk.tolist())}
+    fine = {(l - 1, x >> 1, y >> 1, z >> 1) for l, x, y, z in keys if l > 1}
+    # a block is corrected where the block beside it, at its own level, is refined
+    corrected = np.array([any((l, *np.add((x, y, z), d)) in fine for d in
+                              ((1, 0, 0), (-1, 0, 0), (0, 1, 0), (0, -1, 0), (0, 0, 1), (0, 0, -1)))
+                          for l, (x, y, z) in zip(lev.tolist(), ijk.tolist())])
+    assert corrected.sum() >= 5 and (~corrected).sum() >= 5
+    for part in (corrected, ~corrected):
+        assert np.abs(g[part, 8] - r[part, 8]).sum() < tol * np.abs(r[part, 8]).sum()

@@ -1,11 +1,12 @@
 """HLLC picks the side of the contact before it forms that side's state, flux and star state (in
 packed pairs for the FP32 x/y-faces): parity with the FP64 oracle on flows whose faces take all
 four cases, the fan to either side of the face (supersonic both ways along every axis) and
-either star state, with walls and a refined block."""
+either star state, with walls, on a uniform mesh and with a refined block, whose
+faces' fluxes correct the coarse ones."""
 import numpy as np
 import pytest
 
-from parity_util import TOL_FP64, gpu_mesh, oracle_solver, rel_l1
+from parity_util import TOL_FP64, force_refine, gpu_mesh, oracle_solver, rel_l1
 
 pytestmark = pytest.mark.gpu
 OUT, PER, REF = "outflow", "periodic", "reflect"
@@ -25,12 +26,16 @@ def _fast(x, y, z):
 @pytest.mark.parametrize("rb,tol", [(8, TOL_FP64), (4, 1e-5)])
 @pytest.mark.parametrize("limiter", ["minmod", "vanleer"])
 @pytest.mark.parametrize("bc", [(PER,) * 6, (OUT, OUT, REF, REF, PER, PER)])
-def test_all_sides(rb, tol, limiter, bc):
+@pytest.mark.parametrize("refine", [False, True])
+def test_all_sides(rb, tol, limiter, bc, refine):
     spec = dict(physics="hd", limiter=limiter, flux="hllc", rk=2, base_blocks=(2, 2, 2), max_level=2, bc=bc)
     o = oracle_solver(spec)
     o.set_state(_fast)
     m = gpu_mesh(spec, real_bytes=rb)
     m.set_state(_fast)
+    if refine:
+        force_refine(o, m, {(1, 1, 0, 1)})
+        m.set_state_blocks(o.get_state()[2])
     for _ in range(2):
         dt = o.cfl_dt()
         o.step(dt)
@@ -38,6 +43,7 @@ def test_all_sides(rb, tol, limiter, bc):
     lev, _, g = m.get_state()
     _, _, r = o.get_state()
     m.close()
+    assert set(lev) == ({1, 2} if refine else {1})
     v = r[:, 1:4] / r[:, :1]
     c = np.sqrt(5 / 9 * 2 * np.maximum(r[:, 4] - 0.5 * r[:, 0] * (v ** 2).sum(1), 0) / r[:, 0] * 1.0)
     assert np.all([(v[:, d] / c).max() > 1.2 and (v[:, d] / c).min() < -1.2 for d in range(3)])

@@ -57,6 +57,48 @@ def test_recovery_against_extended_precision(eos, gamma, lorentz, theta):
     assert np.all(np.abs(aux[:, 1] / lor - 1) <= half + 1.5 * lor ** 4 * 1e-12)
 
 
+@pytest.mark.parametrize("eos,gamma", [("ideal", 4.0 / 3.0), ("ideal", 5.0 / 3.0), ("synge", 4.0 / 3.0)])
+@pytest.mark.parametrize("lorentz,theta,branch", [(1.001, (-1, 1), 1), (10.0, (-2, 1), 1), (60.0, (-1, 2), 1),
+                                                  (3.0, (-3.2, -2.2), 1), (3.0, (-5.5, -4.8), 0), (200.0, (0, 1), None)])
+def test_density_and_pressure_against_extended_precision(eos, gamma, lorentz, theta, branch):
+    """The two outputs whose cancellation the guards of the pairs are for. Bound: the FP32 rounding, 2^-29
+    for the pairs, and what the last step's first-order update leaves out (as for xi and Gamma; of rho
+    half of Gamma's and its own, of p through d2p/dxi2 < 4 Gamma^4 / xi). Starts a few roundings off
+    the root, as a step leaves them, and far from it."""
+    rng = np.random.RandomState(12)
+    n = 4096
+    rho = 10 ** rng.uniform(-2, 2, n)
+    u = rng.randn(n, 3)
+    # the upper half of the range of rapidities where the branch is to be that range's
+    lor = np.exp(rng.uniform(np.log(lorentz) * (0.5 if branch is None else 0.0), np.log(lorentz), n))
+    u *= (np.sqrt(lor ** 2 - 1) / np.sqrt((u ** 2).sum(1)))[:, None]
+    th = 10 ** rng.uniform(*theta, n)
+    g = np.sqrt(1 + (u ** 2).sum(1))
+    h = 2.5 * th + np.sqrt(2.25 * th ** 2 + 1) if eos == "synge" else 1 + gamma / (gamma - 1) * th
+    w = rho * h * g
+    cons = np.column_stack([g * rho, w[:, None] * u, g * w - rho * th - g * rho]).astype(np.float32)
+    start = np.float32(g * w) * np.float32(1 + 2.0 ** -21) * np.where(np.arange(n) % 2, np.float32(1), np.float32(1.2))
+    got = agile.recover32(cons, start, gamma, eos)
+    if branch is not None:
+        assert (got[:, 7] == branch).mean() > 0.95, np.unique(got[:, 7], return_counts=True)
+    c = cons.astype(np.float64)
+    xi, lr = _root(c, eos, gamma)
+    D = c[:, 0].astype(np.longdouble)
+    r = D / lr
+    p = xi - (c[:, 4].astype(np.longdouble) + D)
+    ok = got[:, 7] >= 0
+    assert ok.mean() > 0.99 and (ok.all() or branch != 1)
+    ok &= p > 0
+    half, out = 2.0 ** -24 * 1.04, 1e-12 * lr ** 4
+    er, ep = np.abs(got[:, 0] / r - 1), np.abs(got[:, 4] / p - 1)
+    assert np.all((er <= half + 2.0 ** -29 + 2 * out)[ok]), (er / (half + 2.0 ** -29 + 2 * out))[ok].max()
+    assert np.all((ep <= half + 2.0 ** -29 + 2 * out * xi / p)[ok]), (ep / (half + 2.0 ** -29 + 2 * out * xi / p))[ok].max()
+    if lorentz <= 10 and branch == 1:             # rms of a rounding to the nearest: 0.29 ulp
+        for e, v in ((er, r), (ep, p)):
+            ulp = (e * np.abs(v) / np.spacing(np.abs(v).astype(np.float32))).astype(np.float64)
+            assert np.sqrt((ulp ** 2).mean()) <= 0.30
+
+
 @pytest.mark.parametrize("eos,scalar", [("ideal", 4.106e-7), ("synge", 8.375e-7)])
 def test_energy_of_a_cold_gas(eos, scalar):
     """tau = Gamma^2 rho h - p - D cancels in a cold gas: FP32 against FP64 steps from the same state. The

@@ -6,25 +6,16 @@ import numpy as np
 import pytest
 
 from paper_2607_19277_gb300 import agile, workloads as W
+from parity_util import side_by_side, stage_ic
 
 pytestmark = pytest.mark.gpu
 PER, OUT, REF = "periodic", "outflow", "reflect"
 
 
-def _loop(x, y, z):
-    p = np.zeros((7,) + np.shape(x))
-    th = 0.7 * np.sin(2 * np.pi * (x + z))
-    p[0] = 1.0 + 0.3 * np.sin(2 * np.pi * (y - z))
-    p[1] = 0.4 * np.cos(2 * np.pi * z)
-    p[2] = 1.0 + 0.3 * np.cos(2 * np.pi * x)
-    p[4], p[5], p[6] = np.cos(th) * np.cos(0.3 * th), np.sin(th) * np.cos(0.3 * th), np.sin(0.3 * th)
-    return p
-
-
 def _ic(physics):
     if physics == "srhd":   # (prolonging stronger shear leaves states without primitives, in the oracle too)
         return W.srhd_shells(7, 48, n_shells=1, smooth=True, width=4, lorentz_max=2, p_amb=1.0)
-    return _loop if physics == "ffhd_htc" else W.random_smooth(agile.NVAR[agile.PHYSICS[physics]], 5, physics)
+    return stage_ic(physics)
 
 
 def _run(cfgs, physics, flags, steps=2):
@@ -47,13 +38,20 @@ def _run(cfgs, physics, flags, steps=2):
     ("mhd", 4, "hll", "vanleer", (PER,) * 6, False),
     ("srhd", 8, "tvdlf", "minmod", (PER, PER, OUT, OUT, OUT, REF), False),
     ("srhd", 4, "tvdlf", "vanleer", (PER,) * 6, False),
+    ("synge", 8, "tvdlf", "minmod", (PER, PER, OUT, OUT, OUT, REF), False),
+    ("synge", 4, "tvdlf", "vanleer", (PER,) * 6, False),
+    ("ffhd", 8, "tvdlf", "minmod", (PER, PER, PER, PER, OUT, REF), False),
+    ("ffhd", 4, "tvdlf", "vanleer", (PER, PER, PER, PER, REF, OUT), False),
+    ("ffhd_htc", 8, "tvdlf", "vanleer", (PER,) * 6, False),
     ("ffhd_htc", 4, "tvdlf", "vanleer", (PER, PER, PER, PER, REF, OUT), False),
     ("hd", 4, "tvdlf", "minmod", (OUT,) * 6, True),
     ("mhd", 8, "hll", "minmod", (PER,) * 6, True),
     ("srhd", 4, "tvdlf", "vanleer", (PER,) * 6, True),
 ])
 def test_items_give_the_same_bits(physics, rb, flux, limiter, bc, refine):
-    common = dict(physics=physics, limiter=limiter, flux=flux, rk=2, real_bytes=rb,
+    eos = "synge" if physics == "synge" else "ideal"
+    physics = "srhd" if physics == "synge" else physics
+    common = dict(physics=physics, limiter=limiter, flux=flux, rk=2, real_bytes=rb, eos=eos,
                   htc_kappa0=1e-3 if physics == "ffhd_htc" else 0.0)
     cfg = agile.make_config(base_blocks=(2, 1, 3), bc=bc, max_level=2 if refine else 1, **common)
     flags = None
@@ -65,3 +63,10 @@ def test_items_give_the_same_bits(physics, rb, flux, limiter, bc, refine):
         mixed = _run([cfg, agile.make_config(base_blocks=(nx, ny, nz), **common)], physics, flags)
         for a, m in zip(alone, mixed):
             assert np.array_equal(a, m), (nx, ny, nz)
+
+
+@pytest.mark.parametrize("rb", [8, 4])
+def test_items_give_the_same_bits_with_resistivity(rb):
+    alone = side_by_side((1, 1, 1), rb)
+    for reps in ((3, 3, 2), (3, 4, 5), (4, 4, 5), (4, 6, 4)):           # 108 to 576 blocks
+        assert np.array_equal(alone, side_by_side(reps, rb)), reps

@@ -120,6 +120,17 @@ def test_rcp64_selftest_rejects_divisors_outside_its_range(lib, bad):
     assert e.value.status == 1
 
 
+def test_selftests_reject_bad_arguments_on_the_host(lib):
+    import numpy as np
+    from paper_2607_19277_gb300 import agile
+    d, f = np.ones(8), np.ones(8, dtype=np.float32)
+    dp, fp = d.ctypes.data_as(C.POINTER(C.c_double)), f.ctypes.data_as(C.POINTER(C.c_float))
+    for op, n in ((-1, 8), (max(agile.FP64_OPS.values()) + 1, 8), (0, 0), (0, (1 << 26) + 1)):
+        assert lib.agile_selftest_fp64(op, dp, dp, n, None, dp) == 1
+    for eos, gamma, n in ((2, 1.5, 1), (0, 1.0, 1), (0, float("nan"), 1), (0, 1.5, 0)):
+        assert lib.agile_selftest_recover32(eos, gamma, fp, fp, n, None, fp) == 1
+
+
 def test_conduction_config_checked_on_host(lib):
     """ffhd with conduction: TVDLF only, uniform meshes, a finite kappa0 >= 0."""
     from paper_2607_19277_gb300 import agile
