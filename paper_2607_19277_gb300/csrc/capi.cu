@@ -259,8 +259,6 @@ agile_status make_tmap(agile_mesh* m, void* U, CUtensorMap* out) {
   return AGILE_OK;
 }
 
-// (Re)build descriptors, slots and scratch for the current host mesh; U[0] must already
-// hold nblk blocks.
 // 2-D Morton code of (x, y) (16 bits each): the bit strings spread by halves.
 uint64_t morton2(uint32_t x, uint32_t y) {
   auto spread = [](uint32_t v) {
@@ -297,6 +295,8 @@ std::vector<int> slab_order(const HostMesh& hm) {
   return w;
 }
 
+// (Re)build descriptors, slots and scratch for the current host mesh; U[0] must already
+// hold nblk blocks.
 agile_status rebuild(agile_mesh* m) {
   std::vector<BlockDesc> desc;
   std::vector<GhostTask> ghosts;
@@ -371,11 +371,10 @@ agile_status fill_ghosts(agile_mesh* m, void* U) {
   return AGILE_OK;
 }
 
-// Evaluate the initial condition on the listed blocks (host callback, then prim -> cons on
-// the device), in chunks to bound host and device staging.
 // Initial state of the listed blocks: primitives from the mesh's callback at the cell centres,
 // or (prim_src non-null) from the host array prim_src[i][nv][16^3] for the i-th listed
-// block; converted to conserved variables on the device.
+// block; converted to conserved variables on the device, in chunks to bound host and device
+// staging.
 agile_status apply_ic(agile_mesh* m, void* U, const std::vector<int>& blocks, const double* prim_src = nullptr) {
   const int chunk = 256;
   std::vector<double> prim(prim_src ? 0 : (size_t)chunk * m->nv * NCELL);   // callback staging

@@ -1,13 +1,13 @@
 // Device kernels of the block update (sm_103a).
 //
-// stage_kernel is the per-stage macro-kernel (paper Section 2.1.3): one CTA per 16^3
-// block, 256 threads, one thread per (x, y) column marching along z. Per plane it
-// recovers primitives (interior from a per-thread register window, the x/y halo from the
-// neighbours through the block's face table), reconstructs (PLM) and solves the Riemann
-// problem at each x-, y- and z-face ONCE (x/y faces through shared memory, z faces kept
-// in registers between planes), then forms -div F and the SSPRK stage combine. The
-// paper's OpenACC version recomputes each face from both sides; here every face flux is
-// evaluated once.
+// stage_kernel is the per-stage macro-kernel (paper Section 2.1.3): a CTA of 256 threads per
+// work item (a 16^3 block or some planes of one), one thread per (x, y) column marching along z.
+// Per plane it recovers primitives (its own columns from planes the TMA fetches, the x/y halo from
+// the neighbours through the block's face table) into a ring of three planes in shared memory,
+// reconstructs (PLM) and solves the Riemann problem at each x-, y- and z-face ONCE (x/y faces
+// through shared memory, z faces kept in registers between planes), then forms -div F and the
+// SSPRK stage combine. The paper's OpenACC version recomputes each face from both sides; here
+// every face flux is evaluated once.
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -453,10 +453,10 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   // s's barrier.
   __shared__ int s_next;
   __shared__ int s_src[6], s_slot[6];   // face sources / register slots of the current block
-  __shared__ R s_kc[12];                // per-(solve, level) constants, formed by thread 0
+  __shared__ R s_kc[9];                 // per-(solve, level) constants
   // Launch constants, and the per-(solve, level) constants of the current block: they are
   // recomputed only when the block's solve or level differs from the previous block's (a
-  // CTA-uniform test), by one thread.
+  // CTA-uniform test).
   PhysParamsT<R> pp;
   R ra, rb;
   if constexpr (sizeof(R) == 4) {
@@ -517,14 +517,14 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
         const double dxm = fmin(fmin(bd.dx[0], bd.dx[1]), bd.dx[2]);
         fr = R(exp(-0.5 * dtch[0] * dtch[1] * A.glm_alpha / dxm));
       }
-      s_kc[8] = fr;
+      s_kc[5] = fr;
     }
     if (t == 96) {
       PhysParamsT<R> q;
       q.set_ch(dtch[1]);
-      s_kc[9] = q.ch;
-      s_kc[10] = q.ich;
-      s_kc[11] = q.ch2;
+      s_kc[6] = q.ch;
+      s_kc[7] = q.ich;
+      s_kc[8] = q.ch2;
     }
     __syncthreads();
     idx = s_kc[0];
@@ -537,10 +537,10 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
       wz = FU * rdt * idz;
     }
     rq4 = s_kc[4];
-    glm_fr = s_kc[8];
-    pp.ch = s_kc[9];
-    pp.ich = s_kc[10];
-    pp.ch2 = s_kc[11];
+    glm_fr = s_kc[5];
+    pp.ch = s_kc[6];
+    pp.ich = s_kc[7];
+    pp.ch2 = s_kc[8];
     key_sv = sv;
     key_lev = bd.level;
   }
@@ -678,8 +678,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   };
   // States of the face between cells q[o] and q[2 o] of a ring plane (o: the step along the
   // face's direction), from half-slopes of the two cells in shared memory (SHARED_SLOPES; ns
-  // apart per variable) or
-  // formed here.
+  // apart per variable) or formed here.
   auto face_states = [&](const R* q, int o, const R* sl, const R* sr, int ns, R* pl, R* pr) {
     if constexpr (SHARED_SLOPES) {
 #pragma unroll

@@ -23,8 +23,8 @@ enum : int { LIM_MINMOD = 0, LIM_VANLEER = 1 };
 enum : int { FLUX_TVDLF = 0, FLUX_HLL = 1, FLUX_HLLC = 2 };
 enum : int { ST_ENOCONV = 1, ST_EUNPHYS = 2 };
 
-// Equation parameters in the stencil precision R, derived once per CTA (the FP64 copy of
-// gamma serves the SRHD primitive recovery in FP64).
+// Equation parameters in the stencil precision R, formed on the host for a launch (the cleaning
+// speed's per solve in the kernel; the FP64 copy of gamma serves the SRHD primitive recovery in FP64).
 template <typename R>
 struct PhysParamsT {
   double gamma_d, gm_d;    // gamma and (gamma - 1) / gamma in FP64 (SRHD primitive recovery)
@@ -120,7 +120,6 @@ __device__ __forceinline__ double rsqrt_div(double a, double b) {
   return fma(r * y, fma(e, 0.375, 0.5), s);
 }
 __device__ __forceinline__ float rsign(float a) { return copysignf(1.0f, a); }
-__device__ __forceinline__ double rsign(double a) { return copysign(1.0, a); }
 // Reciprocal and quotient in the stencil precision. FP32: the build's fast single-precision
 // divide. FP64: the hardware reciprocal estimate (PTX rcp.approx.ftz.f64) refined by one
 // third-order Newton-Raphson step: with e = 1 - s r0, r1 = r0 (1 + e + e^2) is the series of
@@ -690,10 +689,6 @@ struct SrhdPhysE {
     aux[0] = (R)xi;
     aux[1] = (R)lor;
     if (!(rho > 0.0) || !(pr > 0.0)) st |= ST_EUNPHYS;
-  }
-
-  __device__ static __forceinline__ R enthalpy(R rho, R pres, const PhysParamsT<R>& pp) {
-    return Eos::enthalpy(rdiv(pres, rho), pp);
   }
 
   __device__ static __forceinline__ void prim2cons(const R* p, R* u, const PhysParamsT<R>& pp) {
