@@ -31,7 +31,9 @@ cudaError_t launch_chained(void (*k)(KArgs...), dim3 grid, unsigned block, size_
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...);
+  if (e != cudaSuccess) cudaGetLastError();   // reported here, not by the next launch's check as well
+  return e;
 }
 
 // Per-stage update (macro-kernel), dispatched on physics / precision / limiter / flux.

@@ -43,3 +43,11 @@ def test_chained_kernels_read_kernel_written_memory_with_ordinary_loads():
                     "cooling_kernel"}
     # the halo view's helpers, inlined into the stage kernel
     assert set(re.findall(r"__restrict__\s+(\w+)", texts["kernels.cuh"])) <= TABLES
+
+
+def test_a_failed_chained_launch_leaves_no_error_behind():
+    """A launch by <<< >>> is followed by cudaGetLastError, which reports its error and clears it; the
+    extended launch returns its error and has to clear it as well, or the next launch would report it."""
+    body = _source("launch.h").split("launch_chained(", 1)[1].split("\n}", 1)[0]
+    call = re.search(r"cudaLaunchKernelEx\([^;]*;(.*)", body, re.S)
+    assert call and "cudaGetLastError()" in call.group(1)
