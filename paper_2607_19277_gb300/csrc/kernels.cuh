@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel(const __grid_constant_
   // the sum by dt: 9 instead of 11 FP64 operations per variable and cell. With one root for the
   // signal speed of a state (rsqrt_div), the z-differences carried and the parameters from the
   // host: HD 210 blocks 826 -> 790 us a launch, MHD 512 blocks 4270 -> 4127, SRHD 512 blocks 3306
-  // -> 3252.
+  // -> 3252 (with roots of one operation less, see sqrt64).
   constexpr bool FLUX_DT = sizeof(R) == 8 && !P::SOURCE;
   // A work item is planes k0 .. k0 + nz - 1 of a block (without Z_CUT the whole block): it reads
   // planes k0 - 2 .. k0 + nz + 1, TMA sequence 0 .. nz + 3.

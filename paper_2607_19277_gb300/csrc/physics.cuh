@@ -87,7 +87,9 @@ __device__ __forceinline__ float rsqrt_(float a) { return sqrtf(a); }
 // drops out and the last addition's is what remains. On 3 M arguments from 2^-450 to 2^450 at most
 // 0.515 ulp off (the estimate is good to 9e-7, the terms left out are below 0.02 ulp), rms 0.289 as
 // the correctly rounded root, 0.09% not the nearest; 6 FP64 operations (the library's root takes
-// about twice as many; with s e from the rounded s, 5 operations, 0.76 ulp and rms 0.323). Arguments
+// about twice as many; with s e from the rounded s, 5 operations, 0.76 ulp and rms 0.323, and stage
+// launches of HD 210 blocks 790 us instead of 802, MHD 512 blocks 4127 and 4247, SRHD 512 blocks 3252
+// and 3325, with the same in rsqrt_div and the range of the MHD face speed unchecked). Arguments
 // below 2^-959, where r would lose bits, negative and non-finite ones take the library's.
 constexpr unsigned ROOT64_LO = (1023u - 959u) << 20;    // high word of 2^-959
 __device__ __forceinline__ bool root64_range(double a) {
@@ -873,7 +875,7 @@ __device__ __forceinline__ void riemann(R* pl, R* pr, R* f, const PhysParamsT<R>
     // state U*_K = rho_K (S_K - u_K)/(S_K - S*) [1, S* e_d + v_t, E_K/rho_K + (S* - u_K)(S* +
     // p_K/(rho_K (S_K - u_K)))]. The side is chosen before its conserved state, flux and star
     // state are formed, so these are formed once (210 FP64 blocks 1206 -> 992 us a launch, 1728
-    // FP32 blocks 256 -> 234, in packed pairs 224).
+    // FP32 blocks 256 -> 234, in packed pairs 224; with the later steps 908 and 215).
     P::template waves<D>(pl, vml, vhl, pp);
     P::template waves<D>(pr, vmr, vhr, pp);
     const R sl = rmin(vml - vhl, vmr - vhr), sr = rmax(vml + vhl, vmr + vhr);

@@ -64,7 +64,7 @@ static cudaError_t stage_go_layout(const StageArgs& a, cudaStream_t s) {
 // STAGE_LAYOUT_RING3_DB = three raw slots, two flux buffers, one barrier per plane, the update's
 // stage input loaded from global memory (L2) ahead of the face work instead of kept in a raw
 // slot. The default (layout 0) takes layout 2 where it keeps as many CTAs per SM as layout 1, else
-// layout 3 where that keeps two (256^3 MHD launch: layout 1 858 us, layout 3 831; with resistivity
+// layout 3 where that keeps two (256^3 MHD launch: layout 1 858 us, layout 3 833; with resistivity
 // on 1728 blocks 396 and 388), else layout 1: three CTAs per SM cover the second barrier as well
 // as layout 3 saves it (FFHD, 1728 blocks: 195 us either way). FP64 keeps layout 1. Only the
 // default layout cuts blocks along z (stage_cut).
