@@ -146,12 +146,12 @@ FP64_LANES = 2       # FP64 FMA lanes per SM on GB300 (1.25 TFLOP/s measured at 
 
 
 # DRAM bytes (read + write) per stage launch of the FP32 MHD stage kernel on this workload,
-# from one ncu capture of the three stage launches of one SSPRK3 step (1.201, 1.839 and
-# 1.804 GB; blocks taken in z-slab order), averaged; valid only while the kernel sources
+# from one ncu capture of the three stage launches of one SSPRK3 step (1.1998, 1.8432 and
+# 1.8087 GB; blocks taken in z-slab order), averaged; valid only while the kernel sources
 # hash to STAGE_SRC_DIGEST.
-STAGE_TRAFFIC_BYTES = (1.2008e9 + 1.8389e9 + 1.8044e9) / 3
-STAGE_SRC_DIGEST = "0d29d99aee7755b5"
-STAGE_SRC = ("kernels.cuh", "pair.cuh", "physics.cuh", "stage_go.cuh", "stage_mhd.cu")
+STAGE_TRAFFIC_BYTES = (1.1998e9 + 1.8432e9 + 1.8087e9) / 3
+STAGE_SRC_DIGEST = "127121a679273134"
+STAGE_SRC = ("kernels.cuh", "pair.cuh", "physics.cuh", "stage_cut.h", "stage_go.cuh", "stage_mhd.cu")
 
 
 def stage_traffic():

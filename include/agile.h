@@ -83,9 +83,10 @@ typedef struct {
  *  flux           AGILE_TVDLF (all), AGILE_HLL (hd, mhd), AGILE_HLLC (hd); the
  *                 solvers per module of paper Table 1
  *  rk             2 or 3: SSPRK2 (Heun) or SSPRK3 (Shu-Osher "threestep")
- *  real_bytes     8 (FP64 stencil) or 4 (FP32 stencil; the SRHD primitive recovery in FP64 or,
- *                 where that loses nothing, in pairs of FP32 numbers; FP64 for the time step
- *                 and the conserved sums)
+ *  real_bytes     8 (FP64 stencil) or 4 (FP32 stencil; the last step of the SRHD primitive
+ *                 recovery in pairs of FP32 numbers, some 46 bits, where Gamma and p / xi are
+ *                 such that the results' errors stay those of FP64, else in FP64; FP64 for the
+ *                 time step and the conserved sums)
  *  gamma          ratio of specific heats (ideal gas)
  *  cfl            Courant number: dt = cfl / max_cells sum_d (|v_d| + c_d) / dx_d
  *  glm_alpha      GLM damping parameter alpha (Section 2.3.3; 0.5 in the paper)
